@@ -176,6 +176,7 @@ struct laph_ctx {
     size_t pinned_bytes = 0;
     std::map<std::string, int> tune;   // autotune cache: key -> chosen block size
     int sm_count = 0;
+    int *xg_flag = nullptr;            // mapped host word raised by a tensor-core GEMM whose wait gave up
 };
 
 namespace laph {

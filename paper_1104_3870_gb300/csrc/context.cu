@@ -178,6 +178,7 @@ extern "C" void laph_ctx_destroy(laph_ctx *ctx) {
     for (auto &kv : ctx->ws)
         if (kv.second.ptr) cudaFree(kv.second.ptr);
     if (ctx->pinned) cudaFreeHost(ctx->pinned);
+    if (ctx->xg_flag) cudaFreeHost(ctx->xg_flag);
     delete ctx;
 }
 

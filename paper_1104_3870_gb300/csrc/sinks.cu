@@ -77,7 +77,9 @@ void sinks(const Geom &g, int nv, int nrhs, const c64 *ev, const c64 *sol, c64 *
 
 void sinks_tensor_core(laph_ctx *ctx, const Geom &g, const c64 *V, int nv, const c64 *X, int nrhs, c64 *coef,
                        cudaStream_t s);
-void sinks_tc_check(cudaStream_t s);
+namespace xg {
+void check_host_flag(laph_ctx *ctx);
+}
 
 // LAPH_SINKS_FP64=1 selects the FP64 CUDA-core kernel above instead of the tensor-core one
 // (sinks_tc.cu), for comparisons.
@@ -111,7 +113,8 @@ extern "C" int laph_sinks(laph_ctx *ctx, const laph_lattice *lat, const void *ev
             sinks(g, nv, nrhs, ev, x, (c64 *)o.dev, s);
         } else {
             sinks_tensor_core(ctx, g, ev, nv, x, nrhs, (c64 *)o.dev, s);
-            sinks_tc_check(s);
+            LAPH_CUDA(cudaStreamSynchronize(s));
+            xg::check_host_flag(ctx);
         }
         o.commit(s);
     });
