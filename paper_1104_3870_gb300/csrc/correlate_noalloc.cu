@@ -36,17 +36,91 @@ namespace laph {
 constexpr size_t NOALLOC_SCRATCH_BYTES = 16u << 20;   // 16 MiB per device
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_SCRATCH_BYTES];
 
-// Kernels shared with correlate.cu (same definitions, launched through their host stubs).
+// Kernel shared with correlate.cu (same definition, launched through its host stub).
 struct W4 {
     c64 w[4][4];
 };
 __global__ void rho_at_t0_kernel(int nt, int nv, int nb, int t0, const uint8_t *codes, const uint8_t *mask, c64 *out);
-__global__ void meson_fn_kernel(int nv, int nb, int ntA, int ntB, const c64 *__restrict__ A, const c64 *__restrict__ B,
-                                W4 W, c64 *__restrict__ M);
-__global__ void contract2_kernel(int nt, int nb, int t0, const c64 *Msink, const c64 *Msrc, double scale, c64 *corr);
-__global__ void pipi_p_kernel(int nb, const c64 *S12, const c64 *M32, c64 *P);
+
+// FP64 contractions of this entry point: the tensor-core GEMM of correlate() keeps partial sums in the
+// context's workspace, which this path does not have.
+namespace {
+
+// M[t][b1][b2] = sum_n sum_{a,b} conj(A[b1][tA][a][n]) W[a][b] B[b2][tB][b][n]
+// A, B: [nb][ntA][4][nv]; the slice used is t (or 0 when the operand has a single slice).
+__global__ void meson_fn_kernel(int nv, int nb, int ntA, int ntB, const c64 *__restrict__ A,
+                                const c64 *__restrict__ B, W4 W, c64 *__restrict__ M) {
+    extern __shared__ c64 aw[];   // [4][nv]
+    const int t = blockIdx.x, b1 = blockIdx.y;
+    const int tA = ntA == 1 ? 0 : t, tB = ntB == 1 ? 0 : t;
+    const c64 *a = A + (((long)b1 * ntA + tA) * 4) * nv;
+    for (int e = threadIdx.x; e < 4 * nv; e += blockDim.x) {
+        int bb = e / nv, n = e % nv;
+        c64 s{0, 0};
+#pragma unroll
+        for (int aa = 0; aa < 4; ++aa) s += cmul_conj(a[aa * nv + n], c64{1, 0}) * W.w[aa][bb];
+        aw[bb * nv + n] = s;
+    }
+    __syncthreads();
+    for (int b2 = threadIdx.x; b2 < nb; b2 += blockDim.x) {
+        const c64 *bp = B + (((long)b2 * ntB + tB) * 4) * nv;
+        c64 s{0, 0};
+        for (int e = 0; e < 4 * nv; ++e) s += aw[e] * bp[e];
+        M[((long)t * nb + b1) * nb + b2] = s;
+    }
+}
+
+// corr[dt] (+)= -scale * sum_{b1 b2} Msink[t0+dt][b1][b2] conj(Msrc[b1][b2])
+__global__ void contract2_kernel(int nt, int nb, int t0, const c64 *Msink, const c64 *Msrc, double scale, c64 *corr) {
+    __shared__ c64 sm[256];
+    int dt = blockIdx.x;
+    int t = (t0 + dt) % nt;
+    c64 acc{0, 0};
+    for (int e = threadIdx.x; e < nb * nb; e += blockDim.x)
+        acc += cmul_conj(Msrc[e], Msink[(long)t * nb * nb + e]);
+    sm[threadIdx.x] = acc;
+    __syncthreads();
+    for (int st = blockDim.x / 2; st > 0; st >>= 1) {
+        if ((int)threadIdx.x < st) sm[threadIdx.x] += sm[threadIdx.x + st];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) corr[dt] += (-scale) * sm[0];
+}
+
+// R[t][b1][b4] = sum_{b3} (sum_{b2} conj(S12[b1][b2]) M32[t][b3][b2]) conj(S34[b3][b4])
+__global__ void pipi_p_kernel(int nb, const c64 *S12, const c64 *M32, c64 *P) {
+    int t = blockIdx.x;
+    for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
+        int b1 = e / nb, b3 = e % nb;
+        c64 s{0, 0};
+        for (int b2 = 0; b2 < nb; ++b2) s += cmul_conj(S12[b1 * nb + b2], M32[((long)t * nb + b3) * nb + b2]);
+        P[(long)t * nb * nb + e] = s;
+    }
+}
+
+// X[t] = sum_{b1,b4} M14[t][b1][b4] sum_{b3} P[t][b1][b3] conj(S34[b3][b4]);  corr[dt] = D[dt] - X[t0+dt]
 __global__ void pipi_x_kernel(int nt, int nb, int t0, const c64 *P, const c64 *S34, const c64 *M14, const c64 *cpi12,
-                              const c64 *cpi34, c64 *corr);
+                              const c64 *cpi34, c64 *corr) {
+    __shared__ c64 sm[256];
+    int dt = blockIdx.x;
+    int t = (t0 + dt) % nt;
+    c64 acc{0, 0};
+    for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
+        int b1 = e / nb, b4 = e % nb;
+        c64 r{0, 0};
+        for (int b3 = 0; b3 < nb; ++b3) r += P[(long)t * nb * nb + b1 * nb + b3] * conj(S34[b3 * nb + b4]);
+        acc += M14[(long)t * nb * nb + e] * r;
+    }
+    sm[threadIdx.x] = acc;
+    __syncthreads();
+    for (int st = blockDim.x / 2; st > 0; st >>= 1) {
+        if ((int)threadIdx.x < st) sm[threadIdx.x] += sm[threadIdx.x + st];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) corr[dt] = cpi12[dt] * cpi34[dt] - sm[0];
+}
+
+}  // namespace
 
 // Projector masks computed on the device from the dilution scheme (no host table upload):
 // mask[i][nt + 4 + nv] for the i-th listed projector.

@@ -79,8 +79,23 @@ inline int channel_c(int channel, Mat4 out[3]) {
 // ABI projector masks (correlate.cu) and the diluted noise of each projector at t0
 std::vector<uint8_t> dilution_masks(const laph_dilution &d, int nt, int nv, const int *b_list, int nb);
 __global__ void rho_at_t0_kernel(int nt, int nv, int nb, int t0, const uint8_t *codes, const uint8_t *mask, c64 *out);
-__global__ void meson_fn_kernel(int nv, int nb, int ntA, int ntB, const c64 *__restrict__ A, const c64 *__restrict__ B,
-                                W4 W, c64 *__restrict__ M);
-__global__ void contract2_kernel(int nt, int nb, int t0, const c64 *Msink, const c64 *Msrc, double scale, c64 *corr);
+// Meson functions of one or two row lines with one or two column lines on every slice and at the
+// source (mesonfn_tc.cu): M[z][nl nb][nl nb], z < nt the slices (a, b: [nb][nt][4][nv]) and z = nt the
+// source (ra, rb: [nb][4][nv]); new_lines false where the call before had the same lines.
+struct MesonLines {
+    int nl;
+    const c64 *a[2], *b[2], *ra[2], *rb[2];
+};
+void meson_fns_tc(laph_ctx *ctx, int nt, int nv, int nb, const MesonLines &ln, const Mat4 &W, bool new_lines, c64 *M,
+                  cudaStream_t s);
+// Phi[p][t][n][m] = scale sum_k conj(A[t][n][k]) ph[p][k / 3] B[t][m][k] (mesonfn_tc.cu)
+void overlaps_tc(laph_ctx *ctx, const Geom &g, int nv, int nmom, const c64 *A, const c64 *B, const c64 *ph, c64 scale,
+                 c64 *phi, cudaStream_t s);
+__global__ void meson_contract_kernel(int nt, int nb, int ld, long off, int t0, const c64 *M, double scale, int add,
+                                      c64 *corr);
+namespace xg {
+// throws LAPH_ERR_TIMEOUT if a tensor-core GEMM of the context gave up waiting (after a synchronisation)
+void check_host_flag(laph_ctx *ctx);
+}
 
 }  // namespace laph

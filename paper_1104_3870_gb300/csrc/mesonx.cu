@@ -38,37 +38,6 @@ __global__ void mom_phase_kernel(int ns, int nmom, const int *mom, c64 *ph) {
     ph[(long)p * v3 + i] = c64{cs, sn};
 }
 
-// Phi[p][t][n][n'] = scale sum_k conj(A[t][n][k]) ph[p][k / 3] B[t][n'][k], k = 3 x + c (A = B = V for
-// the plain overlaps).  16 x 16 output tiles, the K sum in shared-memory slabs of 32.
-constexpr int OV_T = 16, OV_K = 32;
-__global__ void __launch_bounds__(256) overlaps_kernel(long V3, int nv, int nt, const c64 *__restrict__ Av,
-                                                       const c64 *__restrict__ Bv, const c64 *__restrict__ ph,
-                                                       c64 scale, c64 *__restrict__ phi) {
-    __shared__ c64 As[OV_T][OV_K + 1], Bs[OV_T][OV_K + 1];
-    const int tx = threadIdx.x % OV_T, ty = threadIdx.x / OV_T;
-    const int n0 = blockIdx.x * OV_T, m0 = blockIdx.y * OV_T;
-    const int t = blockIdx.z % nt, p = blockIdx.z / nt;
-    const long K = 3 * V3;
-    const c64 *at = Av + (long)t * nv * K, *bt = Bv + (long)t * nv * K;
-    const c64 *pp = ph + (long)p * V3;
-    c64 acc{0, 0};
-    for (long k0 = 0; k0 < K; k0 += OV_K) {
-        for (int e = threadIdx.x; e < OV_T * OV_K; e += blockDim.x) {
-            const int r = e / OV_K, kk = e % OV_K;
-            const long k = k0 + kk;
-            const int na = n0 + r, nb = m0 + r;
-            As[r][kk] = (na < nv && k < K) ? conj(at[(long)na * K + k]) : c64{0, 0};
-            Bs[r][kk] = (nb < nv && k < K) ? pp[k / 3] * bt[(long)nb * K + k] : c64{0, 0};
-        }
-        __syncthreads();
-#pragma unroll 8
-        for (int kk = 0; kk < OV_K; ++kk) acc += As[ty][kk] * Bs[tx][kk];
-        __syncthreads();
-    }
-    const int n = n0 + ty, m = m0 + tx;
-    if (n < nv && m < nv) phi[(((long)p * nt + t) * nv + n) * nv + m] = scale * acc;
-}
-
 // One gauge-covariant step of the colour vectors V [nt][nv][V3][3] (Sec. II, the paths of D^(j)):
 // s = +mu: out(x) = U_mu(x) in(x + mu);  s = -mu: out(x) = U_mu(x - mu)^dag in(x - mu);  mu = 1, 2, 3
 // for x, y, z, periodic in space.  U: [V][4][3][3] (the Laplacian's smeared links).
@@ -200,14 +169,13 @@ extern "C" int laph_mom_overlaps(laph_ctx *ctx, const laph_lattice *lat, const v
         mom_phase_kernel<<<dim3(grid_for(g.V3, 256), nmom), 256, 0, s>>>(g.ns, nmom, dmom, ph);
         LAPH_LAUNCH_CHECK();
         StagedOut o = stage_out(ctx, phi, sizeof(c64) * nmom * g.nt * (size_t)nv * nv, "ov:phi");
-        const dim3 grid((nv + OV_T - 1) / OV_T, (nv + OV_T - 1) / OV_T, g.nt * nmom);
         prof_begin("overlaps", s);
-        overlaps_kernel<<<grid, 256, 0, s>>>(g.V3, nv, g.nt, V, V, ph, c64{1.0, 0.0}, (c64 *)o.dev);
-        LAPH_LAUNCH_CHECK();
-        prof_end("overlaps", s, 16.0 * 3 * g.V3 * g.nt * (double)nv * grid.x * nmom,
+        overlaps_tc(ctx, g, nv, nmom, V, V, ph, c64{1.0, 0.0}, (c64 *)o.dev, s);
+        prof_end("overlaps", s, 16.0 * 3 * g.V3 * g.nt * (double)nv + 16.0 * nmom * g.nt * (double)nv * nv,
                  8.0 * nv * (double)nv * 3 * g.V3 * g.nt * nmom);
         o.commit(s);
         LAPH_CUDA(cudaStreamSynchronize(s));
+        xg::check_host_flag(ctx);
     });
 }
 
@@ -245,27 +213,19 @@ extern "C" int correlate_mom(laph_ctx *ctx, const laph_lattice *lat, const laph_
         LAPH_LAUNCH_CHECK();
         StagedOut out = stage_out(ctx, corr, sizeof(c64) * nt, "cm:corr");
         c64 *c = (c64 *)out.dev;
-        LAPH_CUDA(cudaMemsetAsync(c, 0, sizeof(c64) * nt, s));
         Mat4 cs[3];
         const int nc = channel_c(spec->channel, cs);
-        const Mat4 g5g4 = mat_mul(gamma5(), gamma_mat(3));
-        c64 *Msink = (c64 *)ws_get(ctx, "cm:Msink", sizeof(c64) * nt * nb * nb);
-        c64 *Msrc = (c64 *)ws_get(ctx, "cm:Msrc", sizeof(c64) * nb * nb);
-        const int threads = nb < 128 ? 128 : 256;
+        const Mat4 g5g4d = mat_dag(mat_mul(gamma5(), gamma_mat(3)));   // phibar = g5 g4 phi, rhobar = -g5 g4 rho
+        c64 *M = (c64 *)ws_get(ctx, "cm:M", sizeof(c64) * (size_t)(nt + 1) * nb * nb);
+        const MesonLines ml{1, {cf[0], nullptr}, {cf2, nullptr}, {rho[0], nullptr}, {rho2, nullptr}};
         for (int k = 0; k < nc; ++k) {
-            const Mat4 wsink = mat_mul(mat_dag(g5g4), cs[k]);   // phibar = g5 g4 phi
-            const Mat4 wsrc = mat_scale(-1.0, wsink);           // rhobar = -g5 g4 rho
-            meson_fn_kernel<<<dim3(nt, nb), threads, sizeof(c64) * 4 * nv, s>>>(nv, nb, nt, nt, cf[0], cf2,
-                                                                                to_w4(wsink), Msink);
-            LAPH_LAUNCH_CHECK();
-            meson_fn_kernel<<<dim3(1, nb), threads, sizeof(c64) * 4 * nv, s>>>(nv, nb, 1, 1, rho[0], rho2,
-                                                                               to_w4(wsrc), Msrc);
-            LAPH_LAUNCH_CHECK();
-            contract2_kernel<<<nt, 256, 0, s>>>(nt, nb, t0, Msink, Msrc, 1.0 / nc, c);
+            meson_fns_tc(ctx, nt, nv, nb, ml, mat_mul(g5g4d, cs[k]), k == 0, M, s);
+            meson_contract_kernel<<<nt, 256, 0, s>>>(nt, nb, nb, 0, t0, M, 1.0 / nc, k > 0, c);
             LAPH_LAUNCH_CHECK();
         }
         out.commit(s);
         LAPH_CUDA(cudaStreamSynchronize(s));
+        xg::check_host_flag(ctx);
     });
 }
 
@@ -377,10 +337,9 @@ extern "C" int laph_displaced_overlaps(laph_ctx *ctx, const laph_lattice *lat, c
         const double ang = -M_PI * (double)a / g.ns;
         const double cs = std::cos(ang), sn = std::sin(ang);
         StagedOut o = stage_out(ctx, phi, sizeof(c64) * g.nt * (size_t)nv * nv, "do:phi");
-        const dim3 grid((nv + OV_T - 1) / OV_T, (nv + OV_T - 1) / OV_T, g.nt);
-        overlaps_kernel<<<grid, 256, 0, s>>>(g.V3, nv, g.nt, Dj, Dk, ph, c64{cs, sn}, (c64 *)o.dev);
-        LAPH_LAUNCH_CHECK();
+        overlaps_tc(ctx, g, nv, 1, Dj, Dk, ph, c64{cs, sn}, (c64 *)o.dev, s);
         o.commit(s);
         LAPH_CUDA(cudaStreamSynchronize(s));
+        xg::check_host_flag(ctx);
     });
 }
