@@ -7,9 +7,7 @@
 // sides of one site, so spinor loads coalesce and link / clover loads of a
 // site are shared by the warp (broadcast).
 //
-// Links: L64 [parity][mu][cb][3][3] c64;  L32 [parity][mu][cb] 3 float4 holding
-// the first two rows (12 reals) -- the third row of an SU(3) matrix is
-// conj(row0 x row1).  Clover: per site two Hermitian 6x6 chiral blocks
+// Links: L64 [parity][mu][cb][3][3] c64, L32w the same in FP32.  Clover: per site two Hermitian 6x6 chiral blocks
 // (spins {0,1} and {2,3} x colour), packed as 6 real diagonals followed by
 // the 15 complex strictly-lower entries (row-major), 36 reals per block.
 #pragma once
@@ -24,12 +22,8 @@ struct DiracOp {
     double m0, csw, xi;
     double hw[4];            // -1/2 w_mu
     c64 *L64 = nullptr;      // [2][4][Vh][9]
-    float4 *L32 = nullptr;   // [2][4][Vh][3]
-    __nv_bfloat162 *L16 = nullptr;  // [2][4][Vh][6] (12 reals as 6 bf16 pairs)
     double *clov64 = nullptr;  // A       [2][Vh][2][36]
     double *cinv64 = nullptr;  // A^{-1}  [2][Vh][2][36]
-    float *cinv32 = nullptr;   // A^{-1}  [2][Vh][2][36]
-    __nv_bfloat16 *cinv16 = nullptr;  // A^{-1} [2][Vh][2][36]
     // FP32 inner-operator operands in packed form (dslash_f32.cu)
     int *nbr = nullptr;       // [2][Vh][8] neighbour table, sign-folded
     int *order = nullptr;     // [Vh] visiting order of the output sites (z-blocked), see dslash_f32.cu
@@ -38,12 +32,12 @@ struct DiracOp {
     float *C32wA = nullptr;   // [2][Vh][2][72] clover A (full-lattice K for the learned solver)
 };
 
-// Builds nbr, L32w and C32w from L64 and cinv64 (called by prepare_dirac).
+// Builds nbr and order (called by prepare_dirac).
 void prepare_f32_operands(laph_ctx *ctx, DiracOp &op, cudaStream_t s);
 
 // Builds links/clover on the device from ABI links [V][4][3][3] c64 (device pointer).
 DiracOp prepare_dirac(laph_ctx *ctx, const Geom &g, const c64 *links, double m0, double csw, double xi,
-                      cudaStream_t s, bool need_bf16 = false);
+                      cudaStream_t s);
 
 // Kernel modes of the hopping term D_{p pbar} (fused diagonal part):
 enum HopMode {
@@ -54,7 +48,7 @@ enum HopMode {
 };
 
 // Launches the hopping kernel for output parity p on nr right-hand sides.
-// T = double (FP64 links/clover) or float (FP32 compressed links, FP32 clover inverse).
+// T = double (FP64 links/clover) or float (hop_f32).
 template <typename T>
 void hop(const DiracOp &op, int p, HopMode mode, cpx<T> *out, const cpx<T> *in, const cpx<T> *z,
          const cpx<T> *xp, int nr, cudaStream_t s);

@@ -29,29 +29,6 @@ struct LinkLoad<double> {
     }
 };
 
-template <typename T>
-__device__ __forceinline__ void third_row(cpx<T> u[3][3]) {
-    // row2 = conj(row0 x row1)
-    u[2][0] = conj(u[0][1] * u[1][2] - u[0][2] * u[1][1]);
-    u[2][1] = conj(u[0][2] * u[1][0] - u[0][0] * u[1][2]);
-    u[2][2] = conj(u[0][0] * u[1][1] - u[0][1] * u[1][0]);
-}
-
-template <>
-struct LinkLoad<float> {
-    static __device__ __forceinline__ void load(const DiracOp &op, int p, int mu, long cb, c32 u[3][3]) {
-        const float4 *q = op.L32 + (((long)p * 4 + mu) * op.g.Vh + cb) * 3;
-        float4 a = __ldg(q), b = __ldg(q + 1), c = __ldg(q + 2);
-        u[0][0] = {a.x, a.y};
-        u[0][1] = {a.z, a.w};
-        u[0][2] = {b.x, b.y};
-        u[1][0] = {b.z, b.w};
-        u[1][1] = {c.x, c.y};
-        u[1][2] = {c.z, c.w};
-        third_row(u);
-    }
-};
-
 // ------------------------------------------------------------ spin algebra
 // G d for the lower half (d0, d1) of a spinor; colour component c.
 template <typename T>
@@ -148,11 +125,6 @@ template <>
 struct ClovPtr<double> {
     static __device__ __forceinline__ const double *inv(const DiracOp &op) { return op.cinv64; }
 };
-template <>
-struct ClovPtr<float> {
-    static __device__ __forceinline__ const float *inv(const DiracOp &op) { return op.cinv32; }
-};
-
 template <typename T, int MODE>
 __global__ void __launch_bounds__(256) hop_kernel(DiracOp op, int p, cpx<T> *__restrict__ out,
                                                   const cpx<T> *__restrict__ in, const cpx<T> *__restrict__ z,
@@ -294,7 +266,6 @@ void clov_inv_apply(const DiracOp &op, int p, cpx<T> *out, const cpx<T> *in, int
     LAPH_LAUNCH_CHECK();
 }
 template void clov_inv_apply<double>(const DiracOp &, int, c64 *, const c64 *, int, cudaStream_t);
-template void clov_inv_apply<float>(const DiracOp &, int, c32 *, const c32 *, int, cudaStream_t);
 
 // ------------------------------------------------------------ layout conversion
 __global__ void to_eo_kernel(Geom g, const c64 *__restrict__ abi, int first, int nr, c64 *even, c64 *odd) {

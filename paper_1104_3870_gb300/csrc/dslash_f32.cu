@@ -758,31 +758,6 @@ __global__ void nbr_kernel(Geom g, int *nbr) {
     }
 }
 
-__global__ void links_w_kernel(long n4, const c64 *__restrict__ L64, float4 *L32w) {
-    long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= n4 * 9) return;
-    c64 u = L64[idx];
-    L32w[idx] = make_float4((float)u.re, (float)u.re, (float)u.im, (float)u.im);
-}
-
-__global__ void clov_w_kernel(long nblk, const double *__restrict__ cinv64, float *C32w) {
-    long b = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= nblk) return;
-    const double *src = cinv64 + b * CLOV_BLOCK;
-    float *dst = C32w + b * 72;
-    for (int i = 0; i < 6; ++i) {
-        dst[2 * i] = (float)src[i];
-        dst[2 * i + 1] = (float)src[i];
-    }
-    for (int k = 0; k < 15; ++k) {
-        float re = (float)src[6 + 2 * k], im = (float)src[6 + 2 * k + 1];
-        dst[12 + 4 * k] = re;
-        dst[12 + 4 * k + 1] = re;
-        dst[12 + 4 * k + 2] = im;
-        dst[12 + 4 * k + 3] = im;
-    }
-}
-
 // Visiting order of the output sites of the copy-engine-fed hop: z-blocks of bz planes, and inside
 // a block x (half index) fastest, then y, z, t.  The +-t neighbours of consecutive sites are then
 // bz ns^2 / 2 sites apart instead of a whole slice (ns^3 / 2), which keeps a neighbour tile in L2
@@ -817,19 +792,10 @@ void prepare_f32_operands(laph_ctx *ctx, DiracOp &op, cudaStream_t s) {
     const Geom &g = op.g;
     LAPH_REQUIRE(g.Vh < (1L << 31), "lattice too large for 32-bit neighbour indices");
     op.nbr = (int *)ws_get(ctx, "dirac:nbr", sizeof(int) * 16 * g.Vh);
-    op.L32w = (float4 *)ws_get(ctx, "dirac:L32w", sizeof(float4) * 9 * 8 * g.Vh);
-    op.C32w = (float *)ws_get(ctx, "dirac:C32w", sizeof(float) * 144 * 2 * g.Vh);
-    op.C32wA = (float *)ws_get(ctx, "dirac:C32wA", sizeof(float) * 144 * 2 * g.Vh);
     nbr_kernel<<<grid_for(2 * g.Vh, 256), 256, 0, s>>>(g, op.nbr);
     LAPH_LAUNCH_CHECK();
     op.order = (int *)ws_get(ctx, "dirac:order", sizeof(int) * g.Vh);
     order_kernel<<<grid_for(g.Vh, 256), 256, 0, s>>>(g, hop_zblock(g), op.order);
-    LAPH_LAUNCH_CHECK();
-    links_w_kernel<<<grid_for(8 * g.Vh * 9, 256), 256, 0, s>>>(8 * g.Vh, op.L64, op.L32w);
-    LAPH_LAUNCH_CHECK();
-    clov_w_kernel<<<grid_for(4 * g.Vh, 256), 256, 0, s>>>(4 * g.Vh, op.cinv64, op.C32w);
-    LAPH_LAUNCH_CHECK();
-    clov_w_kernel<<<grid_for(4 * g.Vh, 256), 256, 0, s>>>(4 * g.Vh, op.clov64, op.C32wA);
     LAPH_LAUNCH_CHECK();
 }
 
