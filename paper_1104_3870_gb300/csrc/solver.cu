@@ -133,6 +133,21 @@ static InnerStats bicgstab_schur(laph_ctx *ctx, const DiracOp &op, int nr, const
     return st;
 }
 
+// The FP32 inner solve of a block: in one kernel where the lattice is small, else streamed.
+static InnerStats inner_fp32(laph_ctx *ctx, const DiracOp &op, int nr, const c32 *b, c32 *x, double rel_tol, int maxiter,
+                             int check_every, cudaStream_t s) {
+    if (!bicg_small_fits(op, nr)) return bicgstab_schur<float>(ctx, op, nr, b, x, rel_tol, maxiter, check_every, s, "in32");
+    int *d = (int *)ws_get(ctx, "small:stat", sizeof(int) * 2 * nr);
+    bicg_small(ctx, op, nr, b, x, rel_tol, maxiter, d, d + nr, s);
+    int *h = (int *)pinned_get(ctx, sizeof(int) * 2 * nr);
+    LAPH_CUDA(cudaMemcpyAsync(h, d, sizeof(int) * 2 * nr, cudaMemcpyDeviceToHost, s));
+    LAPH_CUDA(cudaStreamSynchronize(s));
+    InnerStats st;
+    st.iters.assign(h, h + nr);
+    st.status.assign(h + nr, h + 2 * nr);
+    return st;
+}
+
 // The same BiCGStab with every Krylov vector stored in BF16 (one complex per bf2) and FP32
 // arithmetic (LAPH_SOLVE_MIXED_BF16); the iterate x is FP32.  nr must be 32, 64, 128 or 256 (the
 // copy-engine-fed stencil).  Rounding each stored vector to 8 significant bits separates the
@@ -357,7 +372,7 @@ void solve_block(laph_ctx *ctx, const DiracOp &op, const c64 *rhs, c64 *sol, int
             c32 *dx = (c32 *)ws_get(ctx, "dc:dx32", sizeof(c32) * nrows * nr);
             mrhs_copy_scaled<double, float>(nrows, nr, scale, re, rin, s);
             double want = std::max(prm.inner_tol, 0.2 * tol / std::max(worst, tol));
-            st = bicgstab_schur<float>(ctx, op, nr, rin, dx, want, budget, prm.check_every, s, "in32");
+            st = inner_fp32(ctx, op, nr, rin, dx, want, budget, prm.check_every, s);
             mrhs_axpy_scaled<float, double>(nrows, nr, scale + nr, dx, xe, s);
         }
         int mx = 0;
