@@ -5,8 +5,9 @@
 // few microseconds each with almost nothing in them: 47 us an iteration on 4^3 x 8 with 8 right-hand
 // sides.  Here four lanes own a site: lane mu takes the forward and backward hop of direction mu, the
 // four partial sums are exchanged by shuffles, and lane mu forms the three components of spin mu.  A
-// lane keeps its components of x, r, p, v, s and t in registers; only the operand of the next hop goes
-// through global memory (L2), between cluster barriers (six an iteration).  Inner products are
+// lane keeps its components of x, r, p, v, s and t in registers; only the operand of the next hop leaves
+// it, through the shared memory of its CTA, which the cluster reads, between cluster barriers (six an
+// iteration).  Inner products are
 // compensated FP32 sums (two floats, 48 bits), over lanes, warps and CTAs in a fixed order, so every
 // CTA of a cluster takes the same decision.
 //
@@ -50,6 +51,35 @@ __device__ __forceinline__ F2 two_add(F2 a, F2 b) {
     return {h, e - (h - s)};
 }
 
+__device__ __forceinline__ F2 two_neg(F2 a) { return {-a.h, -a.l}; }
+__device__ __forceinline__ F2 two_mul(F2 a, F2 b) {
+    const float p = a.h * b.h;
+    const float e = fmaf(a.l, b.h, fmaf(a.h, b.l, fmaf(a.h, b.h, -p)));
+    const float h = p + e;
+    return {h, e - (h - p)};
+}
+__device__ __forceinline__ F2 two_div(F2 a, F2 b) {
+    const float q = a.h / b.h;
+    const F2 r = two_add(a, two_neg(two_mul(F2{q, 0.f}, b)));
+    const float q2 = r.h / b.h;
+    const float h = q + q2;
+    return {h, q2 - (h - q)};
+}
+// complex scalars of the recurrences: the FP64 pipe takes 64 cycles to issue a warp's instruction, and
+// the hundred and fifty of an iteration (three divisions) cost more than its four hops
+struct C2 {
+    F2 re, im;
+};
+__device__ __forceinline__ C2 c2_mul(C2 a, C2 b) {
+    return {two_add(two_mul(a.re, b.re), two_neg(two_mul(a.im, b.im))), two_add(two_mul(a.re, b.im), two_mul(a.im, b.re))};
+}
+__device__ __forceinline__ F2 c2_norm(C2 a) { return two_add(two_mul(a.re, a.re), two_mul(a.im, a.im)); }
+__device__ __forceinline__ C2 c2_div(C2 a, C2 b, F2 bn) {   // bn = |b|^2
+    const C2 n = c2_mul(a, C2{b.re, two_neg(b.im)});
+    return {two_div(n.re, bn), two_div(n.im, bn)};
+}
+__device__ __forceinline__ float2 c2_round(C2 a) { return make_float2(a.re.h, a.im.h); }
+
 struct SmallArgs {
     const int *nbr;          // [2][Vh][8]
     const float4 *L;         // [2][4][Vh][9] (re, re, im, im)
@@ -58,7 +88,6 @@ struct SmallArgs {
     float hws, hwt;
     const c32 *b;            // [Vh][12][nr]
     c32 *x;                  // [Vh][12][nr]
-    float2 *u, *w;           // hop operands on the even and odd sites: [nr][Vh][12]
     double rel_tol;
     int maxiter;
     int *iters, *status;     // [nr]
@@ -72,7 +101,7 @@ __device__ __forceinline__ void hop_half(int mu, const float2 *__restrict__ psi,
     const float4 *q = reinterpret_cast<const float4 *>(psi);
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
-        const float4 v = __ldcg(q + k);   // written by other SMs of the cluster
+        const float4 v = q[k];            // shared memory of a CTA of the cluster
         f[2 * k] = make_float2(v.x, v.y);
         f[2 * k + 1] = make_float2(v.z, v.w);
     }
@@ -114,17 +143,20 @@ __device__ __forceinline__ void hop_half(int mu, const float2 *__restrict__ psi,
     }
 }
 
+// A lane's two hops onto its site from the other parity: operands in the cluster's shared memory, links, weights
+struct HopRef {
+    const float2 *f, *b;
+    const float4 *uf, *ub;
+    float cf, cb;
+};
+
 // Components 3 mu .. 3 mu + 2 of A_pp^{-1} D in at site cb (all four lanes of the site call this)
-__device__ __forceinline__ void hop_site(const SmallArgs &a, int p, int cb, int mu, const float2 *__restrict__ in, float2 out[3]) {
-    const int *nb = a.nbr + ((long)p * a.Vh + cb) * 8;
-    const float w = mu == 3 ? a.hwt : a.hws;
-    const int jf = __ldg(nb + mu), jb = __ldg(nb + 4 + mu);
-    const int nf = jf < 0 ? ~jf : jf, nbk = jb < 0 ? ~jb : jb;
+__device__ __forceinline__ void hop_site(const SmallArgs &a, int p, int cb, int mu, const HopRef &r, float2 out[3]) {
     float2 acc[12];
 #pragma unroll
     for (int k = 0; k < 12; ++k) acc[k] = make_float2(0.f, 0.f);
-    hop_half<true>(mu, in + (long)nf * 12, a.L + (((long)p * 4 + mu) * a.Vh + cb) * 9, jf < 0 ? -w : w, acc);
-    hop_half<false>(mu, in + (long)nbk * 12, a.L + (((long)(1 - p) * 4 + mu) * a.Vh + nbk) * 9, jb < 0 ? -w : w, acc);
+    hop_half<true>(mu, r.f, r.uf, r.cf, acc);
+    hop_half<false>(mu, r.b, r.ub, r.cb, acc);
     // lanes mu and mu ^ 2 keep one chirality each (spins 0, 1 in lanes 0, 1), then sum over mu ^ 1
     float2 x[6];
     const bool up = mu < 2;
@@ -169,14 +201,27 @@ __global__ void __launch_bounds__(T) bicg_small_kernel(const SmallArgs a) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, mu = tid & 3;
     __shared__ F2 wsum[T / 32][SB_NRED];
     __shared__ F2 csum[2][SB_NRED];        // this CTA's sums, double-buffered over reductions
-    __shared__ double tot[SB_NRED];
-    __shared__ float2 coef[3];             // alpha, omega, beta
-    __shared__ int state;                  // 0 running, 1 converged, 2 breakdown
-    float2 *u = a.u + (long)rhs * a.Vh * 12, *w = a.w + (long)rhs * a.Vh * 12;
-
+    __shared__ __align__(16) float2 us[T / 4][12], ws[T / 4][12];   // hop operands on this CTA's even and odd sites
+    __shared__ F2 tot[SB_NRED];
     int cb = rank * (T / 4) + (tid >> 2);
     const bool in = cb < a.Vh;
     if (!in) cb = a.Vh - 1;                // works along with the warp, stores nothing
+    HopRef ho[2];                          // onto the odd sites (from us) and onto the even ones (from ws)
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const int p = 1 - e;
+        const int *nb = a.nbr + ((long)p * a.Vh + cb) * 8;
+        const float wt = mu == 3 ? a.hwt : a.hws;
+        const int jf = __ldg(nb + mu), jb = __ldg(nb + 4 + mu);
+        const int nf = jf < 0 ? ~jf : jf, nk = jb < 0 ? ~jb : jb;
+        float2(*buf)[12] = e == 0 ? us : ws;
+        ho[e].f = cluster.map_shared_rank(&buf[nf % (T / 4)][0], nf / (T / 4));
+        ho[e].b = cluster.map_shared_rank(&buf[nk % (T / 4)][0], nk / (T / 4));
+        ho[e].uf = a.L + (((long)p * 4 + mu) * a.Vh + cb) * 9;
+        ho[e].ub = a.L + (((long)(1 - p) * 4 + mu) * a.Vh + nk) * 9;
+        ho[e].cf = jf < 0 ? -wt : wt;
+        ho[e].cb = jb < 0 ? -wt : wt;
+    }
     int red_no = 0;
     // sums of n reals over the cluster into tot[] (every CTA the same order); two barriers of the cluster
     // bracket it where the caller wants them: `publish` before one, `collect` after it
@@ -199,10 +244,23 @@ __global__ void __launch_bounds__(T) bicg_small_kernel(const SmallArgs a) {
         }
     };
     auto collect = [&](int n) {
-        if (tid < n) {
-            F2 s{0.f, 0.f};
-            for (int q = 0; q < nc; ++q) s = two_add(s, *cluster.map_shared_rank(&csum[red_no & 1][tid], q));
-            tot[tid] = (double)s.h + (double)s.l;
+        if (warp == 0) {   // lane q reads CTA q's sums (at most 16 CTAs)
+            F2 s[SB_NRED];
+#pragma unroll
+            for (int k = 0; k < SB_NRED; ++k) {
+                s[k] = F2{0.f, 0.f};
+                if (k < n && lane < nc) s[k] = *cluster.map_shared_rank(&csum[red_no & 1][k], lane);
+            }
+#pragma unroll
+            for (int k = 0; k < SB_NRED; ++k) {
+                if (k >= n) break;
+#pragma unroll
+                for (int o = 8; o > 0; o >>= 1) {
+                    const F2 t{__shfl_xor_sync(0xffffffffu, s[k].h, o), __shfl_xor_sync(0xffffffffu, s[k].l, o)};
+                    s[k] = two_add(s[k], t);
+                }
+                if (lane == 0) tot[k] = s[k];
+            }
         }
         ++red_no;
         __syncthreads();
@@ -225,10 +283,10 @@ __global__ void __launch_bounds__(T) bicg_small_kernel(const SmallArgs a) {
         return make_float2(y.re, y.im);
     };
     auto cdot = [&](float2 y, float2 z) { return make_float2(fmaf(y.y, z.y, y.x * z.x), fmaf(-y.y, z.x, y.x * z.y)); };
-    auto put = [&](float2 *buf, const float2 *f) {
+    auto put = [&](float2(*buf)[12], const float2 *f) {
         if (in) {
 #pragma unroll
-            for (int c = 0; c < 3; ++c) __stcg(buf + (long)cb * 12 + 3 * mu + c, f[c]);
+            for (int c = 0; c < 3; ++c) buf[tid >> 2][3 * mu + c] = f[c];
         }
     };
 
@@ -244,30 +302,29 @@ __global__ void __launch_bounds__(T) bicg_small_kernel(const SmallArgs a) {
         add_c(0, rdot(code >> (2 * c), r[c]));
         d[2] = two_add(d[2], F2{fmaf(r[c].x, r[c].x, r[c].y * r[c].y), 0.f});
     }
-    put(u, p);
+    put(us, p);
     publish(d, 3);
     cluster.sync();
     collect(3);
-    // scalars live in thread 0 of every CTA
-    c64 rho{tot[0], tot[1]}, alpha{1.0, 0.0};
-    double rr = tot[2];
-    const double stop = a.rel_tol * a.rel_tol * rr;
+    // every thread works the scalars out; state: 0 running, 1 converged, 2 breakdown, 3 no next direction
+    C2 rho{tot[0], tot[1]};
+    float rr = tot[2].h;
+    const float stop = (float)(a.rel_tol * a.rel_tol) * rr;
     int its = 0;
-    if (tid == 0) state = (rr > 0.0 && isfinite(rr) && norm2(rho) > 0.0) ? 0 : rr > 0.0 ? 2 : 1;
-    __syncthreads();
+    int state = (rr > 0.f && isfinite(rr) && c2_norm(rho).h > 0.f) ? 0 : rr > 0.f ? 2 : 1;
     F2 rsum{0.f, 0.f};   // this lane's part of <r, r>, summed with the next <rhat, v>
 
     while (state == 0 && its < a.maxiter) {
         ++its;
         // w = A_oo^{-1} D_oe p
         float2 h[3];
-        hop_site(a, 1, cb, mu, u, h);
-        put(w, h);
+        hop_site(a, 1, cb, mu, ho[0], h);
+        put(ws, h);
         cluster.sync();
         // v = p - A_ee^{-1} D_eo w, <rhat, v>, and <r, r> of the residual the iteration began with
         zero_d(3);
         d[2] = rsum;
-        hop_site(a, 0, cb, mu, w, h);
+        hop_site(a, 0, cb, mu, ho[1], h);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             v[c] = in ? csub(p[c], h[c]) : make_float2(0.f, 0.f);
@@ -276,38 +333,32 @@ __global__ void __launch_bounds__(T) bicg_small_kernel(const SmallArgs a) {
         publish(d, 3);
         cluster.sync();
         collect(3);
-        if (tid == 0) {
-            if (its > 1) rr = tot[2];
-            const c64 dv{tot[0], tot[1]};
-            const double dn = norm2(dv);
-            if (!isfinite(rr))
-                state = 2;
-            else if (its > 1 && rr <= stop)
-                state = 1;
-            else if (!(dn > 0.0) || !isfinite(dn) || dn < 1e-60 * rr * rr)
-                state = 2;
-            else {
-                alpha = c64{(rho.re * dv.re + rho.im * dv.im) / dn, (rho.im * dv.re - rho.re * dv.im) / dn};
-                coef[0] = make_float2((float)alpha.re, (float)alpha.im);
-            }
-        }
-        __syncthreads();
+        if (its > 1) rr = tot[2].h;
+        const C2 dv{tot[0], tot[1]};
+        const F2 dn = c2_norm(dv);
+        if (!isfinite(rr))
+            state = 2;
+        else if (its > 1 && rr <= stop)
+            state = 1;
+        else if (!(dn.h > 0.f) || !isfinite(dn.h))
+            state = 2;
         if (state != 0) {
             if (state == 1) --its;   // converged with the iteration before
             break;
         }
+        const C2 alpha = c2_div(rho, dv, dn);
         // s = r - alpha v (in r)
-        const float2 al = coef[0];
+        const float2 al = c2_round(alpha);
 #pragma unroll
         for (int c = 0; c < 3; ++c) r[c] = cfma(cneg(al), v[c], r[c]);
-        put(u, r);
+        put(us, r);
         cluster.sync();
         // t = M s; <t, s>, <t, t>, <rhat, t>, <rhat, s>
-        hop_site(a, 1, cb, mu, u, h);
-        put(w, h);
+        hop_site(a, 1, cb, mu, ho[0], h);
+        put(ws, h);
         cluster.sync();
         zero_d(7);
-        hop_site(a, 0, cb, mu, w, h);
+        hop_site(a, 0, cb, mu, ho[1], h);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             t[c] = in ? csub(r[c], h[c]) : make_float2(0.f, 0.f);
@@ -319,25 +370,20 @@ __global__ void __launch_bounds__(T) bicg_small_kernel(const SmallArgs a) {
         publish(d, 7);
         cluster.sync();
         collect(7);
-        if (tid == 0) {
-            const double tt = tot[6];
-            c64 om{0.0, 0.0};
-            if (tt > 0.0 && isfinite(tt)) om = c64{tot[0] / tt, tot[1] / tt};   // else s = 0: the half step solved it
-            const c64 rn = c64{tot[4], tot[5]} - om * c64{tot[2], tot[3]};
-            c64 beta{0.0, 0.0};
-            if (norm2(om) > 0.0 && norm2(rn) > 0.0 && isfinite(rn.re) && isfinite(rn.im)) {
-                // (rn / rho)(alpha / omega)
-                const c64 num = rn * alpha, den = rho * om;
-                const double dn = norm2(den);
-                beta = c64{(num.re * den.re + num.im * den.im) / dn, (num.im * den.re - num.re * den.im) / dn};
-            } else
-                state = 3;   // no next direction: done if the residual is small, else a breakdown
-            rho = rn;
-            coef[1] = make_float2((float)om.re, (float)om.im);
-            coef[2] = make_float2((float)beta.re, (float)beta.im);
-        }
-        __syncthreads();
-        const float2 om = coef[1], be = coef[2];
+        const F2 tt = tot[6], zero{0.f, 0.f};
+        C2 omega{zero, zero}, beta{zero, zero};
+        if (tt.h > 0.f && isfinite(tt.h))
+            omega = C2{two_div(tot[0], tt), two_div(tot[1], tt)};   // else s = 0: the half step solved it
+        const C2 ot = c2_mul(omega, C2{tot[2], tot[3]});
+        const C2 rn{two_add(tot[4], two_neg(ot.re)), two_add(tot[5], two_neg(ot.im))};
+        const C2 den = c2_mul(rho, omega);
+        const F2 dq = c2_norm(den);
+        if (dq.h > 0.f && isfinite(dq.h) && (rn.re.h != 0.f || rn.im.h != 0.f) && isfinite(rn.re.h) && isfinite(rn.im.h))
+            beta = c2_div(c2_mul(rn, alpha), den, dq);   // (rn / rho)(alpha / omega)
+        else
+            state = 3;   // done if the residual is small, else a breakdown
+        rho = rn;
+        const float2 om = c2_round(omega), be = c2_round(beta);
         rsum = F2{0.f, 0.f};
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -346,18 +392,14 @@ __global__ void __launch_bounds__(T) bicg_small_kernel(const SmallArgs a) {
             p[c] = cfma(be, cfma(cneg(om), v[c], p[c]), r[c]);
             rsum = two_add(rsum, F2{fmaf(r[c].x, r[c].x, r[c].y * r[c].y), 0.f});
         }
-        put(u, p);
+        put(us, p);
         if (state == 3 || its == a.maxiter) {   // the last residual's norm has no later reduction to go with
             zero_d(1);
             d[0] = rsum;
             publish(d, 1);
             cluster.sync();
             collect(1);
-            if (tid == 0) {
-                const int was = state;
-                state = tot[0] <= stop ? 1 : was == 3 || !isfinite(tot[0]) ? 2 : 0;
-            }
-            __syncthreads();
+            state = tot[0].h <= stop ? 1 : state == 3 || !isfinite(tot[0].h) ? 2 : 0;
             break;
         }
         cluster.sync();
@@ -414,7 +456,7 @@ bool bicg_small_fits(const DiracOp &op, int nr) {
     return small_shape(op.g.Vh, nr, nc, T);
 }
 
-void bicg_small(laph_ctx *ctx, const DiracOp &op, int nr, const c32 *b, c32 *x, double rel_tol, int maxiter, int *iters,
+void bicg_small(const DiracOp &op, int nr, const c32 *b, c32 *x, double rel_tol, int maxiter, int *iters,
                 int *status, cudaStream_t s) {
     SmallArgs a;
     a.nbr = op.nbr;
@@ -426,9 +468,6 @@ void bicg_small(laph_ctx *ctx, const DiracOp &op, int nr, const c32 *b, c32 *x, 
     a.hwt = (float)op.hw[3];
     a.b = b;
     a.x = x;
-    const size_t vb = sizeof(float2) * 12 * op.g.Vh * nr;
-    a.u = (float2 *)ws_get(ctx, "small:u", vb);
-    a.w = (float2 *)ws_get(ctx, "small:w", vb);
     a.rel_tol = rel_tol;
     a.maxiter = maxiter;
     a.iters = iters;

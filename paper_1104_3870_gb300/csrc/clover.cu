@@ -174,7 +174,7 @@ __device__ __forceinline__ MX load_fix(const int4 *__restrict__ fix, long V, int
 __global__ void __launch_bounds__(128) field_kernel(Geom g, const int4 *__restrict__ fix, const int *flag,
                                                     double *__restrict__ F) {
     if (*flag) return;
-    const int s = blockIdx.x * 128 + threadIdx.x;
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= g.V) return;
     const int pl = blockIdx.y;
     const int mu = pl < 3 ? 0 : pl < 5 ? 1 : 2, nu = pl < 3 ? pl + 1 : pl < 5 ? pl - 1 : 3;
@@ -350,9 +350,9 @@ __device__ __forceinline__ bool herm6_inverse(Herm6 &a) {
     return ok;
 }
 
-constexpr int BK_SITES = 32;
 
 // smem [site][2][36] doubles -> FP64 array and FP32 stencil form of the block's sites
+template <int BK_SITES>
 __device__ __forceinline__ void store_blocks(const Geom &g, const double *sm, const unsigned char (*loc)[BK_SITES / 2], long s0,
                                              int ns, double *__restrict__ a64, float *__restrict__ a32) {
     const int nh = ns / 2;
@@ -372,6 +372,7 @@ __device__ __forceinline__ void store_blocks(const Geom &g, const double *sm, co
 // sigma_{mu nu} restricted to chirality h is a Pauli matrix: planes (0,1) and (2,3): -s3 and +-s3,
 // (0,2) and (1,3): s2 and +-s2, (0,3) and (1,2): +-s1 and -s1 (upper sign h = 0), so
 //   A_h = diag + s1 x G1 + s2 x G2 + s3 x G3 with three Hermitian colour matrices.
+template <int BK_SITES>
 __global__ void __launch_bounds__(2 * BK_SITES) blocks_kernel(Geom g, const double *__restrict__ F, double diag,
                                                               double cs, double ct,
                                                               double *__restrict__ clov64, double *__restrict__ cinv64,
@@ -431,7 +432,7 @@ __global__ void __launch_bounds__(2 * BK_SITES) blocks_kernel(Geom g, const doub
     };
     if (is < ns) put();
     __syncthreads();
-    store_blocks(g, sm, loc, s0, ns, clov64, C32wA);
+    store_blocks<BK_SITES>(g, sm, loc, s0, ns, clov64, C32wA);
     if (is < ns) ok = herm6_inverse(a);
     double piv[36];
     if (!ok) herm6_inverse_pivoted(o, piv);
@@ -443,7 +444,7 @@ __global__ void __launch_bounds__(2 * BK_SITES) blocks_kernel(Geom g, const doub
             for (int i = 0; i < 36; ++i) o[i] = piv[i];
     }
     __syncthreads();
-    store_blocks(g, sm, loc, s0, ns, cinv64, C32w);
+    store_blocks<BK_SITES>(g, sm, loc, s0, ns, cinv64, C32w);
 }
 
 // ------------------------------------------------------------------ general links (FP64)
@@ -525,13 +526,18 @@ DiracOp prepare_dirac(laph_ctx *ctx, const Geom &g, const c64 *links, double m0,
     LAPH_CUDA(cudaMemsetAsync(flag, 0, sizeof(int), s));
     pack_kernel<<<grid_for(g.V, PK_SITES), 256, 0, s>>>(g, links, op.L64, op.L32w, fix, flag);
     LAPH_LAUNCH_CHECK();
-    field_kernel<<<dim3(grid_for(g.V, 128), 6), 128, 0, s>>>(g, fix, flag, F);
+    // small lattices: short blocks, so that the work reaches more SMs
+    const bool few = g.V < 32 * 2 * 152;
+    const int fb = few ? 32 : 128;
+    field_kernel<<<dim3(grid_for(g.V, fb), 6), fb, 0, s>>>(g, fix, flag, F);
     LAPH_LAUNCH_CHECK();
     field_general_kernel<<<dim3(grid_for(g.V, 64, 512), 6), 64, 0, s>>>(g, links, flag, F);
     LAPH_LAUNCH_CHECK();
-    blocks_kernel<<<grid_for(g.V, BK_SITES), 2 * BK_SITES, 0, s>>>(g, F, diag, -0.5 * csw / xi,
-                                                                  -0.25 * csw * (1.0 + 1.0 / xi), op.clov64, op.cinv64,
-                                                                  op.C32wA, op.C32w);
+    const double cs = -0.5 * csw / xi, ct = -0.25 * csw * (1.0 + 1.0 / xi);
+    if (few)
+        blocks_kernel<8><<<grid_for(g.V, 8), 16, 0, s>>>(g, F, diag, cs, ct, op.clov64, op.cinv64, op.C32wA, op.C32w);
+    else
+        blocks_kernel<32><<<grid_for(g.V, 32), 64, 0, s>>>(g, F, diag, cs, ct, op.clov64, op.cinv64, op.C32wA, op.C32w);
     LAPH_LAUNCH_CHECK();
     prepare_f32_operands(ctx, op, s);
     return op;

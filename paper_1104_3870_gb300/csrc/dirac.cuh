@@ -81,6 +81,10 @@ bool hop_bf16_xpay_dots(laph_ctx *ctx, const DiracOp &op, int p, __nv_bfloat162 
 template <typename T>
 void clov_inv_apply(const DiracOp &op, int p, cpx<T> *out, const cpx<T> *in, int nr, cudaStream_t s);
 
+// out = A_pp^{-1} in in FP64 with red[r] = <out, out>
+void clov_inv_norm(laph_ctx *ctx, const DiracOp &op, int p, cpx<double> *out, const cpx<double> *in, int nr,
+                   cpx<double> *red, cudaStream_t s);
+
 // ABI full-lattice fields [nrhs][V][12] c64 <-> internal parity halves [Vh][12][nr].
 // `first` selects the first right-hand side of the block, `nr` the block size.
 void fields_to_eo(const Geom &g, const c64 *abi, int first, int nr, c64 *even, c64 *odd, cudaStream_t s);

@@ -215,11 +215,15 @@ double hop_bytes(const DiracOp &op, HopMode mode, int nr, size_t real_bytes) {
 // hopping term) + 504 (two 6x6 complex clover blocks).
 double hop_flops(const DiracOp &op, int nr) { return (double)op.g.Vh * nr * 1824.0; }
 
+// Threads per block of a kernel bound by the FP64 pipe of the SMs it runs on: one warp where blocks of
+// four would leave SMs without work (4^3 x 8, 8 right-hand sides: 64 warps, 56 us in blocks of 128).
+static int fp64_block(long n) { return n < 128l * 2 * 152 ? 32 : 128; }
+
 template <typename T>
 void hop(const DiracOp &op, int p, HopMode mode, cpx<T> *out, const cpx<T> *in, const cpx<T> *z, const cpx<T> *xp,
          int nr, cudaStream_t s) {
     long n = op.g.Vh * nr;
-    const int block = 128;
+    const int block = fp64_block(n);
     unsigned grid = grid_for(n, block);
     prof_begin("dslash_fp64", s);
     switch (mode) {
@@ -262,10 +266,50 @@ __global__ void clov_inv_kernel(DiracOp op, int p, cpx<T> *out, const cpx<T> *in
 template <typename T>
 void clov_inv_apply(const DiracOp &op, int p, cpx<T> *out, const cpx<T> *in, int nr, cudaStream_t s) {
     long n = op.g.Vh * nr;
-    clov_inv_kernel<T><<<grid_for(n, 128), 128, 0, s>>>(op, p, out, in, nr);
+    const int block = fp64_block(n);
+    clov_inv_kernel<T><<<grid_for(n, block), block, 0, s>>>(op, p, out, in, nr);
     LAPH_LAUNCH_CHECK();
 }
 template void clov_inv_apply<double>(const DiracOp &, int, c64 *, const c64 *, int, cudaStream_t);
+
+// out = A_pp^{-1} in with <out, out> of every right-hand side: a block holds rpb sites of all nr
+// right-hand sides, sums its sites in FP64 and writes one partial sum per right-hand side.
+__global__ void clov_inv_norm_kernel(DiracOp op, int p, c64 *__restrict__ out, const c64 *__restrict__ in, int nr, int rpb,
+                                     c64 *__restrict__ partial) {
+    extern __shared__ double nsm[];
+    const int r = threadIdx.x % nr, row0 = threadIdx.x / nr;
+    double acc = 0.0;
+    for (long cb = (long)blockIdx.x * rpb + row0; cb < op.g.Vh; cb += (long)gridDim.x * rpb) {
+        c64 x[12], y[12];
+        const c64 *src = in + cb * 12 * nr + r;
+#pragma unroll
+        for (int k = 0; k < 12; ++k) x[k] = src[(long)k * nr];
+        const double *ci = op.cinv64 + ((long)p * op.g.Vh + cb) * 2 * CLOV_BLOCK;
+        herm6<double, double>(ci, x, y);
+        herm6<double, double>(ci + CLOV_BLOCK, x + 6, y + 6);
+        c64 *dst = out + cb * 12 * nr + r;
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+            dst[(long)k * nr] = y[k];
+            acc = fma(y[k].re, y[k].re, fma(y[k].im, y[k].im, acc));
+        }
+    }
+    nsm[threadIdx.x] = acc;
+    __syncthreads();
+    for (int st = rpb / 2; st > 0; st >>= 1) {
+        if (row0 < st) nsm[threadIdx.x] += nsm[threadIdx.x + st * nr];
+        __syncthreads();
+    }
+    if (row0 == 0) partial[(long)blockIdx.x * nr + r] = c64{nsm[r], 0.0};
+}
+
+void clov_inv_norm(laph_ctx *ctx, const DiracOp &op, int p, c64 *out, const c64 *in, int nr, c64 *red, cudaStream_t s) {
+    const RedPlan pl = red_plan(ctx, op.g.Vh, nr);
+    c64 *partial = (c64 *)ws_get(ctx, "red:partial", sizeof(c64) * pl.grid * nr);
+    clov_inv_norm_kernel<<<pl.grid, pl.block, sizeof(double) * pl.block, s>>>(op, p, out, in, nr, pl.rpb, partial);
+    LAPH_LAUNCH_CHECK();
+    red_final_sum(partial, (int)pl.grid, 1, nr, red, s);
+}
 
 // ------------------------------------------------------------ layout conversion
 __global__ void to_eo_kernel(Geom g, const c64 *__restrict__ abi, int first, int nr, c64 *even, c64 *odd) {

@@ -138,7 +138,7 @@ static InnerStats inner_fp32(laph_ctx *ctx, const DiracOp &op, int nr, const c32
                              int check_every, cudaStream_t s) {
     if (!bicg_small_fits(op, nr)) return bicgstab_schur<float>(ctx, op, nr, b, x, rel_tol, maxiter, check_every, s, "in32");
     int *d = (int *)ws_get(ctx, "small:stat", sizeof(int) * 2 * nr);
-    bicg_small(ctx, op, nr, b, x, rel_tol, maxiter, d, d + nr, s);
+    bicg_small(op, nr, b, x, rel_tol, maxiter, d, d + nr, s);
     int *h = (int *)pinned_get(ctx, sizeof(int) * 2 * nr);
     LAPH_CUDA(cudaMemcpyAsync(h, d, sizeof(int) * 2 * nr, cudaMemcpyDeviceToHost, s));
     LAPH_CUDA(cudaStreamSynchronize(s));
@@ -255,8 +255,14 @@ void solve_block(laph_ctx *ctx, const DiracOp &op, const c64 *rhs, c64 *sol, int
     // ||b||^2 of the full field
     mrhs_dots<double>(ctx, pl, nrows, 2, be, be, bo, bo, nullptr, nullptr, red, s);
     std::vector<c64> h_red(3 * nr);
-    LAPH_CUDA(cudaMemcpyAsync(h_red.data(), red, sizeof(c64) * 2 * nr, cudaMemcpyDeviceToHost, s));
-    LAPH_CUDA(cudaStreamSynchronize(s));
+    // sums to the host, through pinned memory: a pageable copy costs another 10 us of host time each
+    auto fetch = [&](int n) {
+        c64 *h = (c64 *)pinned_get(ctx, sizeof(c64) * 3 * nr);
+        LAPH_CUDA(cudaMemcpyAsync(h, red, sizeof(c64) * n, cudaMemcpyDeviceToHost, s));
+        LAPH_CUDA(cudaStreamSynchronize(s));
+        std::copy(h, h + n, h_red.begin());
+    };
+    fetch(2 * nr);
     std::vector<double> bnorm(nr);
     for (int k = 0; k < nr; ++k) bnorm[k] = std::sqrt(h_red[k].re + h_red[nr + k].re);
     // a right-hand side that is not finite cannot be solved: it is reported as not converged
@@ -279,8 +285,6 @@ void solve_block(laph_ctx *ctx, const DiracOp &op, const c64 *rhs, c64 *sol, int
         double worst = 0.0;
         if (cyc == 0) {
             // x = 0: r = b, x_o = A_oo^{-1} b_o, and the Schur residual is bhat itself
-            LAPH_CUDA(cudaMemcpyAsync(xo, to, hb, cudaMemcpyDeviceToDevice, s));
-            LAPH_CUDA(cudaMemcpyAsync(re, bh, hb, cudaMemcpyDeviceToDevice, s));
             for (int k = 0; k < nr; ++k) {
                 rel[k] = rel_of(k, bnorm[k]);
                 if (!bad[k] && rel[k] > tol) {
@@ -288,7 +292,11 @@ void solve_block(laph_ctx *ctx, const DiracOp &op, const c64 *rhs, c64 *sol, int
                     worst = 1.0;
                 }
             }
-            if (all) break;
+            if (all) {
+                LAPH_CUDA(cudaMemcpyAsync(xo, to, hb, cudaMemcpyDeviceToDevice, s));
+                break;
+            }
+            mrhs_dots<double>(ctx, pl, nrows, 1, bh, bh, nullptr, nullptr, nullptr, nullptr, red, s);
         } else {
             // x_o = A_oo^{-1} b_o - A_oo^{-1} D_oe x_e, then the true residual r = b - K x.  With
             // x_o rebuilt this way r_o = b_o - A_oo x_o - D_oe x_e vanishes up to rounding, so a
@@ -300,9 +308,7 @@ void solve_block(laph_ctx *ctx, const DiracOp &op, const c64 *rhs, c64 *sol, int
             for (;;) {
                 mrhs_dots<double>(ctx, pl, nrows, with_ro ? 2 : 1, re, re, with_ro ? ro : nullptr,
                                   with_ro ? ro : nullptr, nullptr, nullptr, red, s);
-                LAPH_CUDA(cudaMemcpyAsync(h_red.data(), red, sizeof(c64) * (with_ro ? 2 : 1) * nr,
-                                          cudaMemcpyDeviceToHost, s));
-                LAPH_CUDA(cudaStreamSynchronize(s));
+                fetch((with_ro ? 2 : 1) * nr);
                 if (with_ro) break;
                 bool stop = cyc == max_outer || total_iters >= prm.maxiter;
                 if (!stop) {
@@ -335,12 +341,10 @@ void solve_block(laph_ctx *ctx, const DiracOp &op, const c64 *rhs, c64 *sol, int
             }
             if (all || cyc == max_outer || total_iters >= prm.maxiter) break;
             // With x_o reconstructed from x_e the Schur residual bhat - M x_e equals A_ee^{-1} r_e.
-            clov_inv_apply<double>(op, 0, tmp, re, nr, s);
-            LAPH_CUDA(cudaMemcpyAsync(re, tmp, hb, cudaMemcpyDeviceToDevice, s));
+            clov_inv_norm(ctx, op, 0, tmp, re, nr, red, s);
         }
-        mrhs_dots<double>(ctx, pl, nrows, 1, re, re, nullptr, nullptr, nullptr, nullptr, red, s);
-        LAPH_CUDA(cudaMemcpyAsync(h_red.data(), red, sizeof(c64) * nr, cudaMemcpyDeviceToHost, s));
-        LAPH_CUDA(cudaStreamSynchronize(s));
+        const c64 *rs = cyc == 0 ? bh : tmp;   // the Schur residual
+        fetch(nr);
         for (int k = 0; k < nr; ++k) {
             double rn = std::sqrt(h_red[k].re);
             bool done = rel[k] <= tol || handed[k] || bad[k] || !(rn > 0.0) || !std::isfinite(rn);
@@ -348,13 +352,15 @@ void solve_block(laph_ctx *ctx, const DiracOp &op, const c64 *rhs, c64 *sol, int
             h_scale[nr + k] = done ? 0.0 : rn;    // back into x_e
             if (!done) outer[k] += 1;
         }
-        LAPH_CUDA(cudaMemcpyAsync(scale, h_scale.data(), sizeof(double) * 2 * nr, cudaMemcpyHostToDevice, s));
+        double *hs = (double *)pinned_get(ctx, sizeof(double) * 2 * nr);
+        std::copy(h_scale.begin(), h_scale.end(), hs);
+        LAPH_CUDA(cudaMemcpyAsync(scale, hs, sizeof(double) * 2 * nr, cudaMemcpyHostToDevice, s));
         int budget = std::max(1, prm.maxiter - total_iters);
         InnerStats st;
         if (prm.mode == LAPH_SOLVE_PLAIN_FP64) {
             c64 *rin = (c64 *)ws_get(ctx, "dc:rin", hb);
             c64 *dx = (c64 *)ws_get(ctx, "dc:dx", hb);
-            mrhs_copy_scaled<double, double>(nrows, nr, scale, re, rin, s);
+            mrhs_copy_scaled<double, double>(nrows, nr, scale, rs, rin, s);
             // ask the inner solve for what the true residual still needs (Schur and true residuals
             // differ by the clover factor, hence the margin)
             double want = std::max(1e-15, 0.2 * tol / std::max(worst, tol));
@@ -363,14 +369,14 @@ void solve_block(laph_ctx *ctx, const DiracOp &op, const c64 *rhs, c64 *sol, int
         } else if (prm.mode == LAPH_SOLVE_MIXED_BF16 && bf16_block_ok(nr)) {
             bf2 *rin = (bf2 *)ws_get(ctx, "dc:rin16", sizeof(bf2) * nrows * nr);
             c32 *dx = (c32 *)ws_get(ctx, "dc:dx32", sizeof(c32) * nrows * nr);
-            mrhs_copy_scaled_bf16(nrows, nr, scale, re, rin, s);
+            mrhs_copy_scaled_bf16(nrows, nr, scale, rs, rin, s);
             double want = std::max(prm.inner_tol, 0.2 * tol / std::max(worst, tol));
             st = bicgstab_schur_bf16(ctx, op, nr, rin, dx, want, budget, prm.check_every, s);
             mrhs_axpy_scaled<float, double>(nrows, nr, scale + nr, dx, xe, s);
         } else {
             c32 *rin = (c32 *)ws_get(ctx, "dc:rin32", sizeof(c32) * nrows * nr);
             c32 *dx = (c32 *)ws_get(ctx, "dc:dx32", sizeof(c32) * nrows * nr);
-            mrhs_copy_scaled<double, float>(nrows, nr, scale, re, rin, s);
+            mrhs_copy_scaled<double, float>(nrows, nr, scale, rs, rin, s);
             double want = std::max(prm.inner_tol, 0.2 * tol / std::max(worst, tol));
             st = inner_fp32(ctx, op, nr, rin, dx, want, budget, prm.check_every, s);
             mrhs_axpy_scaled<float, double>(nrows, nr, scale + nr, dx, xe, s);
@@ -385,7 +391,7 @@ void solve_block(laph_ctx *ctx, const DiracOp &op, const c64 *rhs, c64 *sol, int
     }
     // re, ro hold the true residual b - K x of the current (xe, xo) here: every exit from the
     // cycle loop after cycle 0 comes right after it is computed, and cycle 0 exits only when
-    // every right-hand side is zero.
+    // every right-hand side is zero or not finite (which the fallback leaves out).
     bool need = false;
     for (int k = 0; k < nr; ++k) need |= !(rel[k] <= tol);
     if (prm.fallback && need) {

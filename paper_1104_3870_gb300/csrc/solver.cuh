@@ -14,8 +14,8 @@ void solve_block(laph_ctx *ctx, const DiracOp &op, const c64 *rhs, c64 *sol, int
 // lattice and block are small enough that it is the faster form, and the solve (x = 0 start, device
 // iters / status per right-hand side: 0 budget spent, 1 converged, 2 breakdown).
 bool bicg_small_fits(const DiracOp &op, int nr);
-void bicg_small(laph_ctx *ctx, const DiracOp &op, int nr, const c32 *b, c32 *x, double rel_tol, int maxiter, int *iters,
-                int *status, cudaStream_t s);
+void bicg_small(const DiracOp &op, int nr, const c32 *b, c32 *x, double rel_tol, int maxiter, int *iters, int *status,
+                cudaStream_t s);
 
 // Same contract with FP64 defect correction around FP32 flexible GCR preconditioned by the
 // network of weights (device pointer, layout of laph_precond_train).
