@@ -270,12 +270,8 @@ void bicg_xr_update_reduce(laph_ctx *ctx, const RedPlan &pl, long nrows, const B
                   7.0 * nrows * pl.nr * sizeof(cpx<T>));
 }
 
-template void bicg_p_update<float>(long, int, const BicgScalars &, const c32 *, c32 *, const c32 *, cudaStream_t);
 template void bicg_p_update<double>(long, int, const BicgScalars &, const c64 *, c64 *, const c64 *, cudaStream_t);
-template void bicg_s_update<float>(long, int, const BicgScalars &, const c32 *, const c32 *, c32 *, cudaStream_t);
 template void bicg_s_update<double>(long, int, const BicgScalars &, const c64 *, const c64 *, c64 *, cudaStream_t);
-template void bicg_xr_update_reduce<float>(laph_ctx *, const RedPlan &, long, const BicgScalars &, c32 *, const c32 *,
-                                           const c32 *, const c32 *, c32 *, const c32 *, c64 *, cudaStream_t);
 template void bicg_xr_update_reduce<double>(laph_ctx *, const RedPlan &, long, const BicgScalars &, c64 *, const c64 *,
                                             const c64 *, const c64 *, c64 *, const c64 *, c64 *, cudaStream_t);
 
@@ -420,47 +416,6 @@ void mrhs_rhat_init(laph_ctx *ctx, const RedPlan &pl, long nrows, const c32 *r, 
     rhat_pack_kernel<<<grid_for(nsite * pl.nr, 256), 256, 0, s>>>(nsite, pl.nr, r, code);
     LAPH_LAUNCH_CHECK();
     mrhs_rhat_dots(ctx, pl, nrows, r, code, red, s);
-}
-
-struct XRGenBody {
-    BicgScalars sc;
-    c32 *x;
-    const c32 *p, *sv, *t;
-    c32 *r;
-    const uint32_t *code;
-    int nr;
-    using Acc = c32;
-    __device__ void operator()(long i, int k, Acc *acc) const {
-        const c32 a = cvt<float>(sc.alpha[k]), w = cvt<float>(sc.omega[k]);
-        const c32 si = sv[i];
-        x[i] = x[i] + a * p[i] + w * si;
-        const c32 rn = si - w * t[i];
-        r[i] = rn;
-        acc[0] += rhat_conj_mul(rhat_code_at(code, i, nr), rn);
-        acc[1] += cmul_conj(rn, rn);
-    }
-    __device__ void two(long i, long j, int k, Acc *acc) const {
-        const c32 a = cvt<float>(sc.alpha[k]), w = cvt<float>(sc.omega[k]);
-        const c32 xi = x[i], pi = p[i], si = sv[i], ti = t[i];
-        const c32 xj = x[j], pj = p[j], sj = sv[j], tj = t[j];
-        const uint32_t qi = rhat_code_at(code, i, nr), qj = rhat_code_at(code, j, nr);
-        const c32 ri = si - w * ti, rj = sj - w * tj;
-        x[i] = xi + a * pi + w * si;
-        x[j] = xj + a * pj + w * sj;
-        r[i] = ri;
-        r[j] = rj;
-        acc[0] += rhat_conj_mul(qi, ri);
-        acc[1] += cmul_conj(ri, ri);
-        acc[0] += rhat_conj_mul(qj, rj);
-        acc[1] += cmul_conj(rj, rj);
-    }
-};
-void bicg_xr_update_reduce_gen(laph_ctx *ctx, const RedPlan &pl, long nrows, const BicgScalars &sc, c32 *x,
-                               const c32 *p, const c32 *sv, const c32 *t, c32 *r, const uint32_t *code, c64 *red,
-                               cudaStream_t s) {
-    // read x, p, s, t and the codes; write x, r
-    run_reduce<2>(ctx, pl, nrows, XRGenBody{sc, x, p, sv, t, r, code, pl.nr}, red, s, nullptr,
-                  (6.0 * sizeof(c32) + 4.0 / 12.0) * nrows * pl.nr);
 }
 
 __device__ __forceinline__ c64 cdiv(c64 a, c64 b) {

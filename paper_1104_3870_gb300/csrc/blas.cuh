@@ -103,10 +103,6 @@ void mrhs_rhat_init(laph_ctx *ctx, const RedPlan &pl, long nrows, const cpx<floa
 // red[0][r] = <rhat, v>, red[1][r] = <v, v> for the stored codes
 void mrhs_rhat_dots(laph_ctx *ctx, const RedPlan &pl, long nrows, const cpx<float> *v, const uint32_t *code,
                     c64 *red, cudaStream_t s);
-// x += alpha p + omega s; r = s - omega t; red = <rhat, r>, <r, r> with the coded rhat (FP32)
-void bicg_xr_update_reduce_gen(laph_ctx *ctx, const RedPlan &pl, long nrows, const BicgScalars &sc, cpx<float> *x,
-                               const cpx<float> *p, const cpx<float> *sv, const cpx<float> *t, cpx<float> *r,
-                               const uint32_t *code, c64 *red, cudaStream_t s);
 void bicg_alpha(int nr, const BicgScalars &sc, const c64 *red, cudaStream_t s);
 void bicg_omega(int nr, const BicgScalars &sc, const c64 *red, cudaStream_t s);
 void bicg_rho(int nr, const BicgScalars &sc, const c64 *red, cudaStream_t s);

@@ -56,18 +56,18 @@ void hop(const DiracOp &op, int p, HopMode mode, cpx<T> *out, const cpx<T> *in, 
 // FP32 hop with the packed operands of prepare_f32_operands (modes HOP_CLOVINV and HOP_CLOVINV_XPAY).
 // Throws LAPH_ERR_TIMEOUT (and clears the flag) when a TMA-fed stencil launch gave up waiting for a copy.
 void hop_timeout_check(cudaStream_t s);
+// `live` (may be null): a device word; at zero the kernel returns at once.
 void hop_f32(const DiracOp &op, int p, HopMode mode, cpx<float> *out, const cpx<float> *in, const cpx<float> *z,
-             int nr, cudaStream_t s);
-// The xpay hop out = z - A_pp^{-1} D in with the inner products <out, z> and <out, out> of every
-// right-hand side fused into its epilogue: red[0][r] = <out, z>, red[1][r] = <out, out>.
-// Returns false (launching nothing) where the fused form is not available for this shape.
+             int nr, cudaStream_t s, const int *live = nullptr);
+// The xpay hop out = z - A_pp^{-1} D in with inner products of every right-hand side fused into its
+// epilogue (rcode [Vh][nr]: the coded shadow vector rhat of blas.cuh): <out, z>, <out, out>, <rhat, out>,
+// <rhat, z>, or <rhat, out> alone.  Returns false (launching nothing) where the fused form is not
+// available for this shape.
+struct PartSums;
 bool hop_f32_xpay_dots(laph_ctx *ctx, const DiracOp &op, int p, cpx<float> *out, const cpx<float> *in,
-                       const cpx<float> *z, int nr, cpx<double> *red, cudaStream_t s);
-
-// The same with <rhat, out> (the coded shadow vector of blas.cuh, rcode [Vh][nr] packed words) fused
-// instead: red[0][r] = <rhat, out>.
+                       const cpx<float> *z, int nr, const uint32_t *rcode, const int *live, PartSums *sums, cudaStream_t s);
 bool hop_f32_xpay_rdot(laph_ctx *ctx, const DiracOp &op, int p, cpx<float> *out, const cpx<float> *in,
-                       const cpx<float> *z, int nr, const uint32_t *rcode, cpx<double> *red, cudaStream_t s);
+                       const cpx<float> *z, int nr, const uint32_t *rcode, const int *live, PartSums *sums, cudaStream_t s);
 
 // BF16-stored spinors ([cb][12][nr] bf162: one complex per element), FP32 links and clover inverse, FP32
 // arithmetic: the copy-engine-fed kernel of hop_f32 reading and writing BF16 tiles.  nr must be 32, 64,

@@ -20,7 +20,7 @@
 
 #include <cstdlib>
 
-#include "blas.cuh"
+#include "bicg_f32.cuh"
 #include "dirac.cuh"
 #include "tma.cuh"
 
@@ -147,7 +147,8 @@ template <int MODE>
 __global__ void __launch_bounds__(128, MODE == HOP_APPLY ? 6 : 8) hop2_kernel(const int *__restrict__ nbr, const float4 *__restrict__ L,
                                                    const float *__restrict__ C, long Vh, int p, float hws, float hwt,
                                                    float2 *__restrict__ out, const float2 *__restrict__ in,
-                                                   const float2 *__restrict__ z, int nr) {
+                                                   const float2 *__restrict__ z, int nr, const int *__restrict__ live) {
+    if (live && *live == 0) return;
     long tid = (long)blockIdx.x * blockDim.x + threadIdx.x;
     long cb = tid / nr;
     int r = (int)(tid - cb * nr);
@@ -245,15 +246,20 @@ constexpr long long HOP3_WAIT_CYCLES = 1LL << 31;   // about one second at the m
 
 __device__ int g_hop3_timeout;   // set when a copy wait gives up (or the ring is misaligned); read by the host
 
-// DOTS (xpay mode, nr = 32 RPT): the epilogue also accumulates, per right-hand side, the inner
-// products <out, z> and <out, out> of the warp's sites in FP32 and writes them as the warp's
-// partial sums partial[warp][k][r] (k = 0, 1; FP64) for a fixed-order final sum.
+// DOTS (xpay mode, one right-hand side per lane): the epilogue also accumulates, per right-hand side,
+// inner products of the warp's sites in FP32 and writes them as the warp's partial sums
+// partial[warp][k][lane] for a fixed-order final sum: 1: <out, z>, <out, out>; 2: <rhat, out>;
+// 3: <out, z>, <out, out>, <rhat, out>, <rhat, z>, with rhat the coded shadow vector.  A warp's units
+// all belong to the same 32 right-hand sides (h = warp mod 2^gshift), as gridDim * HOP3_WARPS is a
+// multiple of 2^gshift for up to 128 right-hand sides.
+constexpr int hop3_nred(int dots) { return dots == 1 ? 2 : dots == 2 ? 1 : dots == 3 ? 4 : 0; }
 template <int MODE, int NS, int RPT, int DOTS = 0, typename E = float2, int HPJ = 1>
 __global__ void __launch_bounds__(HOP3_WARPS * 32, HOP3_MINB)
     hop3_kernel(const __grid_constant__ CUtensorMap tm_in, const __grid_constant__ CUtensorMap tm_z,
                 const int *__restrict__ nbr, const int *__restrict__ order, const float4 *__restrict__ L,
                 const float *__restrict__ C, int Vh, int p, float hws, float hwt, E *__restrict__ out, int nr, int gshift,
-                int nunits, c64 *__restrict__ partial, const uint32_t *__restrict__ rcode) {
+                int nunits, float2 *__restrict__ partial, const uint32_t *__restrict__ rcode, const int *__restrict__ live) {
+    if (live && *live == 0) return;   // every right-hand side of the solve has converged
     extern __shared__ __align__(128) unsigned char sm3[];
     constexpr bool CJ = hop3_cj<MODE, HPJ>();
     constexpr int HOP3_SPIN = Hop3Geo<RPT, E, HPJ, CJ>::SPIN, HOP3_SLOT = Hop3Geo<RPT, E, HPJ, CJ>::SLOT;
@@ -353,20 +359,14 @@ __global__ void __launch_bounds__(HOP3_WARPS * 32, HOP3_MINB)
     };
 
     for (int k = 0; k < NS; ++k) issue();
-    float2 dts[RPT];
-    float dtt[RPT];
-#pragma unroll
-    for (int q = 0; q < RPT; ++q) {
-        dts[q] = ff(0.f, 0.f);
-        dtt[q] = 0.f;
-    }
+    static_assert(DOTS == 0 || RPT == 1, "fused products: one right-hand side per lane");
+    float2 dts = ff(0.f, 0.f), drt = ff(0.f, 0.f), drs = ff(0.f, 0.f);
+    float dtt = 0.f;
     bool ok = true;
     for (int k = 0, q = gw; k < nu && ok; ++k, q += gstride) {
         const int cb = __ldg(order + (q >> gshift)), h = q & gmask;
         // packed shadow-vector codes, fetched before the hops so that their latency is hidden
-        uint32_t rw[RPT];
-#pragma unroll
-        for (int q = 0; q < RPT; ++q) rw[q] = DOTS == 2 ? __ldg(rcode + (long)cb * nr + 32 * q + lane) : 0u;
+        const uint32_t rw = DOTS >= 2 ? __ldg(rcode + (long)cb * nr + 32 * h + lane) : 0u;
         float2 acc[RPT][12];
 #pragma unroll
         for (int q = 0; q < RPT; ++q)
@@ -448,15 +448,21 @@ __global__ void __launch_bounds__(HOP3_WARPS * 32, HOP3_MINB)
                     for (int c = 0; c < 12; ++c) {
                         const float2 zc = to_f2(zs[c * 32 * RPT]);
                         res[q][c] = sub2(zc, res[q][c]);
-                        if (DOTS == 1) {   // conj(t) z and |t|^2
-                            const float2 t = res[q][c];
-                            dts[q].x = fmaf(t.x, zc.x, fmaf(t.y, zc.y, dts[q].x));
-                            dts[q].y = fmaf(t.x, zc.y, fmaf(-t.y, zc.x, dts[q].y));
-                            dtt[q] = fmaf(t.x, t.x, fmaf(t.y, t.y, dtt[q]));
-                        } else if (DOTS == 2) {   // conj(rhat) t with the coded shadow vector (nr = 32 RPT)
-                            const c32 v = rhat_conj_mul((rw[q] >> (2 * c)) & 3u, c32{res[q][c].x, res[q][c].y});
-                            dts[q].x += v.re;
-                            dts[q].y += v.im;
+                        const float2 t = res[q][c];
+                        if (DOTS == 1 || DOTS == 3) {   // conj(t) z and |t|^2
+                            dts.x = fmaf(t.x, zc.x, fmaf(t.y, zc.y, dts.x));
+                            dts.y = fmaf(t.x, zc.y, fmaf(-t.y, zc.x, dts.y));
+                            dtt = fmaf(t.x, t.x, fmaf(t.y, t.y, dtt));
+                        }
+                        if (DOTS >= 2) {                // conj(rhat) t, conj(rhat) z
+                            const c32 v = rhat_conj_mul((rw >> (2 * c)) & 3u, c32{t.x, t.y});
+                            drt.x += v.re;
+                            drt.y += v.im;
+                        }
+                        if (DOTS == 3) {
+                            const c32 v = rhat_conj_mul((rw >> (2 * c)) & 3u, c32{zc.x, zc.y});
+                            drs.x += v.re;
+                            drs.y += v.im;
                         }
                     }
                 }
@@ -471,12 +477,16 @@ __global__ void __launch_bounds__(HOP3_WARPS * 32, HOP3_MINB)
         }
     }
     if (DOTS != 0) {   // every warp writes, zeros where it had no units
-        const int gwarp = blockIdx.x * HOP3_WARPS + warp;
-#pragma unroll
-        for (int q = 0; q < RPT; ++q) {
-            const int r = 32 * q + lane;
-            partial[((long)gwarp * 2 + 0) * nr + r] = c64{(double)dts[q].x, (double)dts[q].y};
-            partial[((long)gwarp * 2 + 1) * nr + r] = c64{(double)dtt[q], 0.0};
+        float2 *o = partial + (long)(blockIdx.x * HOP3_WARPS + warp) * hop3_nred(DOTS) * 32 + lane;
+        if (DOTS == 2) {
+            o[0] = drt;
+        } else {
+            o[0] = dts;
+            o[32] = ff(dtt, 0.f);
+            if (DOTS == 3) {
+                o[64] = drt;
+                o[96] = drs;
+            }
         }
     }
     if (!ok) {
@@ -519,9 +529,9 @@ static CUtensorMap spinor_map(const E *base, long Vh, int nr, int rpt) {
 }
 
 template <int MODE, int NS, int RPT, int DOTS = 0, typename E = float2>
-static long launch_hop3(const DiracOp &op, int p, float hws, float hwt, E *out, const E *in,
-                        const E *z, int nr, cudaStream_t s, laph_ctx *ctx = nullptr, c64 *red = nullptr,
-                        const uint32_t *rcode = nullptr) {
+static PartSums launch_hop3(const DiracOp &op, int p, float hws, float hwt, E *out, const E *in,
+                            const E *z, int nr, cudaStream_t s, laph_ctx *ctx = nullptr,
+                            const uint32_t *rcode = nullptr, const int *live = nullptr) {
     // one RHS per lane: two hops per job (the slot still leaves room for four blocks per SM)
     constexpr int HPJ = RPT == 1 ? 2 : 1;
     constexpr size_t smem = (size_t)HOP3_WARPS * NS * (Hop3Geo<RPT, E, HPJ, hop3_cj<MODE, HPJ>()>::SLOT + 8 + 8);
@@ -546,16 +556,14 @@ static long launch_hop3(const DiracOp &op, int p, float hws, float hwt, E *out, 
     long grid = (nunits + HOP3_WARPS - 1) / HOP3_WARPS;
     const long cap = (long)bpsm[dev] * nsm[dev];
     if (grid > cap) grid = cap;
-    c64 *partial = nullptr;
-    if (DOTS != 0) partial = (c64 *)ws_get(ctx, "hop3:dots", sizeof(c64) * 2 * nr * grid * HOP3_WARPS);
+    constexpr int K = hop3_nred(DOTS);
+    float2 *partial = nullptr;
+    if (DOTS != 0) partial = (float2 *)ws_get(ctx, "hop3:dots", sizeof(float2) * K * 32 * grid * HOP3_WARPS);
     hop3_kernel<MODE, NS, RPT, DOTS, E, HPJ><<<(unsigned)grid, HOP3_WARPS * 32, smem, s>>>(
         tin, tz, op.nbr, op.order, op.L32w, MODE == HOP_APPLY ? op.C32wA : op.C32w, (int)op.g.Vh, p, hws, hwt, out, nr,
-        gshift, (int)nunits, partial, rcode);
-    if (DOTS != 0) {
-        LAPH_LAUNCH_CHECK();
-        red_final_sum(partial, (int)(grid * HOP3_WARPS), 2, nr, red, s);
-    }
-    return grid * HOP3_WARPS;
+        gshift, (int)nunits, partial, rcode, live);
+    LAPH_LAUNCH_CHECK();
+    return PartSums{partial, (int)(grid * HOP3_WARPS) >> gshift, (long)(K * 32) << gshift, 32, true};
 }
 
 // Ring depth per warp of the TMA-fed kernel.  Two slots measured fastest on a 16^3 x 32
@@ -583,13 +591,13 @@ static int hop3_rpt_max() {
 
 template <int NS, int RPT>
 static void hop3_modes(const DiracOp &op, int p, HopMode mode, float hws, float hwt, float2 *out, const float2 *in,
-                       const float2 *z, int nr, cudaStream_t s) {
+                       const float2 *z, int nr, cudaStream_t s, const int *live) {
     if (mode == HOP_APPLY)
-        launch_hop3<HOP_APPLY, NS, RPT>(op, p, hws, hwt, out, in, z, nr, s);
+        launch_hop3<HOP_APPLY, NS, RPT>(op, p, hws, hwt, out, in, z, nr, s, nullptr, nullptr, live);
     else if (mode == HOP_CLOVINV)
-        launch_hop3<HOP_CLOVINV, NS, RPT>(op, p, hws, hwt, out, in, (const float2 *)nullptr, nr, s);
+        launch_hop3<HOP_CLOVINV, NS, RPT>(op, p, hws, hwt, out, in, (const float2 *)nullptr, nr, s, nullptr, nullptr, live);
     else
-        launch_hop3<HOP_CLOVINV_XPAY, NS, RPT>(op, p, hws, hwt, out, in, z, nr, s);
+        launch_hop3<HOP_CLOVINV_XPAY, NS, RPT>(op, p, hws, hwt, out, in, z, nr, s, nullptr, nullptr, live);
 }
 
 void hop_timeout_check(cudaStream_t s) {
@@ -607,7 +615,8 @@ void hop_timeout_check(cudaStream_t s) {
 double hop_bytes(const DiracOp &op, HopMode mode, int nr, size_t real_bytes);
 double hop_flops(const DiracOp &op, int nr);
 
-void hop_f32(const DiracOp &op, int p, HopMode mode, c32 *out, const c32 *in, const c32 *z, int nr, cudaStream_t s) {
+void hop_f32(const DiracOp &op, int p, HopMode mode, c32 *out, const c32 *in, const c32 *z, int nr, cudaStream_t s,
+             const int *live) {
     LAPH_REQUIRE(mode == HOP_CLOVINV || mode == HOP_CLOVINV_XPAY || mode == HOP_APPLY,
                  "FP32 hop supports the clover-inverse and apply modes");
     long n = op.g.Vh * nr;
@@ -625,58 +634,52 @@ void hop_f32(const DiracOp &op, int p, HopMode mode, c32 *out, const c32 *in, co
         const float2 *i = (const float2 *)in, *zz = (const float2 *)z;
         const bool two = hop3_rpt_max() == 2 && nr % 64 == 0;
         if (ns == 3)
-            two ? hop3_modes<3, 2>(op, p, mode, hws, hwt, o, i, zz, nr, s)
-                : hop3_modes<3, 1>(op, p, mode, hws, hwt, o, i, zz, nr, s);
+            two ? hop3_modes<3, 2>(op, p, mode, hws, hwt, o, i, zz, nr, s, live)
+                : hop3_modes<3, 1>(op, p, mode, hws, hwt, o, i, zz, nr, s, live);
         else
-            two ? hop3_modes<2, 2>(op, p, mode, hws, hwt, o, i, zz, nr, s)
-                : hop3_modes<2, 1>(op, p, mode, hws, hwt, o, i, zz, nr, s);
-    } else if (mode == HOP_APPLY)
+            two ? hop3_modes<2, 2>(op, p, mode, hws, hwt, o, i, zz, nr, s, live)
+                : hop3_modes<2, 1>(op, p, mode, hws, hwt, o, i, zz, nr, s, live);
+    } else {
+        if (mode == HOP_APPLY)
         hop2_kernel<HOP_APPLY><<<grid, block, 0, s>>>(op.nbr, op.L32w, op.C32wA, op.g.Vh, p, hws, hwt, (float2 *)out,
-                                                      (const float2 *)in, (const float2 *)z, nr);
+                                                      (const float2 *)in, (const float2 *)z, nr, live);
     else if (mode == HOP_CLOVINV)
         hop2_kernel<HOP_CLOVINV><<<grid, block, 0, s>>>(op.nbr, op.L32w, op.C32w, op.g.Vh, p, hws, hwt, (float2 *)out,
-                                                        (const float2 *)in, (const float2 *)z, nr);
+                                                        (const float2 *)in, (const float2 *)z, nr, live);
     else
         hop2_kernel<HOP_CLOVINV_XPAY><<<grid, block, 0, s>>>(op.nbr, op.L32w, op.C32w, op.g.Vh, p, hws, hwt,
-                                                             (float2 *)out, (const float2 *)in, (const float2 *)z, nr);
-    LAPH_LAUNCH_CHECK();
+                                                             (float2 *)out, (const float2 *)in, (const float2 *)z, nr, live);
+        LAPH_LAUNCH_CHECK();
+    }
     prof_end("dslash_fp32", s, hop_bytes(op, mode, nr, sizeof(float)), hop_flops(op, nr));
 }
 
-bool hop_f32_xpay_dots(laph_ctx *ctx, const DiracOp &op, int p, c32 *out, const c32 *in, const c32 *z, int nr,
-                       c64 *red, cudaStream_t s) {
+// One right-hand side per lane: with two the fused epilogue spills registers.
+static bool dots_shape(const DiracOp &op, const void *in, const void *z, int nr) {
     const bool aligned = ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(z) |
                            reinterpret_cast<uintptr_t>(op.L32w) | reinterpret_cast<uintptr_t>(op.C32w)) & 15) == 0;
-    const int ns = hop3_stages();
-    const int rpt = (hop3_rpt_max() == 2 && nr == 64) ? 2 : 1;
-    if (!aligned || ns != 2 || nr != 32 * rpt) return false;
-    float hws = (float)op.hw[0], hwt = (float)op.hw[3];
+    return aligned && hop3_stages() == 2 && (nr == 32 || nr == 64 || nr == 128) && op.g.Vh * (nr / 32) < (1L << 30);
+}
+
+bool hop_f32_xpay_dots(laph_ctx *ctx, const DiracOp &op, int p, c32 *out, const c32 *in, const c32 *z, int nr,
+                       const uint32_t *rcode, const int *live, PartSums *sums, cudaStream_t s) {
+    if (!dots_shape(op, in, z, nr)) return false;
+    const float hws = (float)op.hw[0], hwt = (float)op.hw[3];
     prof_begin("dslash_fp32", s);
-    if (rpt == 2)
-        launch_hop3<HOP_CLOVINV_XPAY, 2, 2, 1>(op, p, hws, hwt, (float2 *)out, (const float2 *)in,
-                                                  (const float2 *)z, nr, s, ctx, red);
-    else
-        launch_hop3<HOP_CLOVINV_XPAY, 2, 1, 1>(op, p, hws, hwt, (float2 *)out, (const float2 *)in,
-                                                  (const float2 *)z, nr, s, ctx, red);
-    LAPH_LAUNCH_CHECK();
-    prof_end("dslash_fp32", s, hop_bytes(op, HOP_CLOVINV_XPAY, nr, sizeof(float)), hop_flops(op, nr));
+    *sums = launch_hop3<HOP_CLOVINV_XPAY, 2, 1, 3>(op, p, hws, hwt, (float2 *)out, (const float2 *)in, (const float2 *)z,
+                                                   nr, s, ctx, rcode, live);
+    prof_end("dslash_fp32", s, hop_bytes(op, HOP_CLOVINV_XPAY, nr, sizeof(float)) + (double)op.g.Vh * 4 * nr,
+             hop_flops(op, nr));
     return true;
 }
 
-// The xpay hop out = z - A_pp^{-1} D in with <rhat, out> of every right-hand side fused into its
-// epilogue (rhat the coded shadow vector of blas.cuh, rcode[cb][r] packed words): red[0][r] = <rhat, out>,
-// red[1][r] = 0.
 bool hop_f32_xpay_rdot(laph_ctx *ctx, const DiracOp &op, int p, c32 *out, const c32 *in, const c32 *z, int nr,
-                       const uint32_t *rcode, c64 *red, cudaStream_t s) {
-    // one right-hand side per lane only: with two the fused epilogue spills registers
-    const bool aligned = ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(z) |
-                           reinterpret_cast<uintptr_t>(op.L32w) | reinterpret_cast<uintptr_t>(op.C32w)) & 15) == 0;
-    if (!aligned || hop3_stages() != 2 || nr != 32) return false;
-    float hws = (float)op.hw[0], hwt = (float)op.hw[3];
+                       const uint32_t *rcode, const int *live, PartSums *sums, cudaStream_t s) {
+    if (!dots_shape(op, in, z, nr)) return false;
+    const float hws = (float)op.hw[0], hwt = (float)op.hw[3];
     prof_begin("dslash_fp32", s);
-    launch_hop3<HOP_CLOVINV_XPAY, 2, 1, 2>(op, p, hws, hwt, (float2 *)out, (const float2 *)in, (const float2 *)z, nr,
-                                           s, ctx, red, rcode);
-    LAPH_LAUNCH_CHECK();
+    *sums = launch_hop3<HOP_CLOVINV_XPAY, 2, 1, 2>(op, p, hws, hwt, (float2 *)out, (const float2 *)in, (const float2 *)z,
+                                                   nr, s, ctx, rcode, live);
     prof_end("dslash_fp32", s, hop_bytes(op, HOP_CLOVINV_XPAY, nr, sizeof(float)) + (double)op.g.Vh * 4 * nr,
              hop_flops(op, nr));
     return true;
@@ -719,20 +722,35 @@ void hop_bf16(const DiracOp &op, int p, HopMode mode, __nv_bfloat162 *out, const
     else
         two ? (void)launch_hop3<HOP_CLOVINV_XPAY, 2, 2, 0>(op, p, hws, hwt, out, in, z, nr, s)
             : (void)launch_hop3<HOP_CLOVINV_XPAY, 2, 1, 0>(op, p, hws, hwt, out, in, z, nr, s);
-    LAPH_LAUNCH_CHECK();
     prof_end("dslash_bf16", s, hop_bytes_bf16(op, mode, nr), hop_flops(op, nr));
+}
+
+// red[k][r] = sum over the items of value k, one block per (k, r), fixed order
+__global__ void parts_final_kernel(PartSums ps, int K, int nr, c64 *red) {
+    __shared__ c64 sm[256];
+    const int k = blockIdx.x / nr, r = blockIdx.x % nr;
+    const float2 *p = (const float2 *)ps.p + (long)(r >> 5) * ps.kstride * K + (r & 31) + k * ps.kstride;
+    c64 a{0.0, 0.0};
+    for (int i = threadIdx.x; i < ps.count; i += 256) {
+        const float2 z = p[i * ps.istride];
+        a += c64{(double)z.x, (double)z.y};
+    }
+    sm[threadIdx.x] = a;
+    __syncthreads();
+    for (int st = 128; st > 0; st >>= 1) {
+        if ((int)threadIdx.x < st) sm[threadIdx.x] += sm[threadIdx.x + st];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) red[blockIdx.x] = sm[0];
 }
 
 bool hop_bf16_xpay_dots(laph_ctx *ctx, const DiracOp &op, int p, __nv_bfloat162 *out, const __nv_bfloat162 *in,
                         const __nv_bfloat162 *z, int nr, c64 *red, cudaStream_t s) {
-    const int rpt = (hop3_rpt_max() == 2 && nr == 64) ? 2 : 1;
-    if (!bf16_ok(op, in, z, nr) || nr != 32 * rpt) return false;
+    if (!bf16_ok(op, in, z, nr) || nr > 64) return false;
     const float hws = (float)op.hw[0], hwt = (float)op.hw[3];
     prof_begin("dslash_bf16", s);
-    if (rpt == 2)
-        launch_hop3<HOP_CLOVINV_XPAY, 2, 2, 1>(op, p, hws, hwt, out, in, z, nr, s, ctx, red);
-    else
-        launch_hop3<HOP_CLOVINV_XPAY, 2, 1, 1>(op, p, hws, hwt, out, in, z, nr, s, ctx, red);
+    const PartSums ps = launch_hop3<HOP_CLOVINV_XPAY, 2, 1, 1>(op, p, hws, hwt, out, in, z, nr, s, ctx);
+    parts_final_kernel<<<2 * nr, 256, 0, s>>>(ps, 2, nr, red);
     LAPH_LAUNCH_CHECK();
     prof_end("dslash_bf16", s, hop_bytes_bf16(op, HOP_CLOVINV_XPAY, nr), hop_flops(op, nr));
     return true;

@@ -9,10 +9,9 @@
 // the full operator.
 #include <algorithm>
 #include <cmath>
-#include <type_traits>
 #include <vector>
 
-#include "blas.cuh"
+#include "bicg_f32.cuh"
 #include "dirac.cuh"
 #include "solver.cuh"
 
@@ -31,37 +30,9 @@ static void schur_apply(const DiracOp &op, int nr, const cpx<T> *in, cpx<T> *out
     hop<T>(op, 0, HOP_CLOVINV_XPAY, out, tmp_o, in, nullptr, nr, s);        // out = in - A_ee^{-1} D_eo tmp
 }
 
-// t = M s and the two inner products <t, s>, <t, t> into red[0..1][r]; in FP32 the products
-// come out of the epilogue of the second hop where that form exists.
-template <typename T>
-static void schur_apply_tdots(laph_ctx *ctx, const RedPlan &pl, long nrows, const DiracOp &op, int nr,
-                              const cpx<T> *sv, cpx<T> *t, cpx<T> *tmp_o, c64 *red, cudaStream_t s) {
-    hop<T>(op, 1, HOP_CLOVINV, tmp_o, sv, nullptr, nullptr, nr, s);
-    if (std::is_same<T, float>::value &&
-        hop_f32_xpay_dots(ctx, op, 0, (c32 *)t, (const c32 *)tmp_o, (const c32 *)sv, nr, red, s))
-        return;
-    hop<T>(op, 0, HOP_CLOVINV_XPAY, t, tmp_o, sv, nullptr, nr, s);
-    mrhs_dots<T>(ctx, pl, nrows, 2, t, sv, t, t, nullptr, nullptr, red, s);
-}
-
-// BiCGStab on the Schur operator for nr right-hand sides at once, x = 0 start.
-// Per-RHS relative stopping on the recursive residual; host polls every
-// `check_every` iterations (device-side scalars, no per-iteration sync).
-template <typename T>
-static InnerStats bicgstab_schur(laph_ctx *ctx, const DiracOp &op, int nr, const cpx<T> *b, cpx<T> *x,
-                                 double rel_tol, int maxiter, int check_every, cudaStream_t s,
-                                 const std::string &tag) {
-    const Geom &g = op.g;
-    long nrows = g.Vh * 12;
-    size_t vb = sizeof(cpx<T>) * nrows * nr;
-    auto V = [&](const char *n) { return (cpx<T> *)ws_get(ctx, tag + n, vb); };
-    // FP32: the shadow vector is the rounded phase of r0 stored as packed 2-bit codes (blas.cuh),
-    // and <rhat, v> comes out of the stencil's epilogue; FP64 (the plain solver): rhat = r0, stored
-    constexpr bool gen = std::is_same<T, float>::value;
-    cpx<T> *r = V(":r"), *rh = gen ? nullptr : V(":rh"), *p = V(":p"), *v = V(":v"), *sv = V(":s"), *t = V(":t");
-    cpx<T> *tmp = V(":tmp");
-    uint32_t *rc = gen ? (uint32_t *)ws_get(ctx, tag + ":rc", sizeof(uint32_t) * (size_t)(nrows / 12) * nr) : nullptr;
-    char *scb = (char *)ws_get(ctx, tag + ":sc", (sizeof(c64) * 4 + sizeof(double) * 2 + sizeof(int) * 3) * nr + 256);
+// Device scalars of a solve (one allocation) and their host mirror.
+static BicgScalars scalars_get(laph_ctx *ctx, const std::string &name, int nr) {
+    char *scb = (char *)ws_get(ctx, name, (sizeof(c64) * 4 + sizeof(double) * 2 + sizeof(int) * 3) * nr + 256);
     BicgScalars sc;
     sc.rho = (c64 *)scb;
     sc.alpha = sc.rho + nr;
@@ -72,80 +43,127 @@ static InnerStats bicgstab_schur(laph_ctx *ctx, const DiracOp &op, int nr, const
     sc.active = (int *)(sc.rr_stop + nr);
     sc.status = sc.active + nr;
     sc.iters = sc.status + nr;
-    c64 *red = (c64 *)ws_get(ctx, tag + ":red", sizeof(c64) * 3 * nr);
+    return sc;
+}
+
+static InnerStats stats_fetch(laph_ctx *ctx, const int *iters, const int *status, int nr, cudaStream_t s) {
+    int *h = (int *)pinned_get(ctx, sizeof(int) * 2 * nr);
+    LAPH_CUDA(cudaMemcpyAsync(h, iters, sizeof(int) * nr, cudaMemcpyDeviceToHost, s));
+    LAPH_CUDA(cudaMemcpyAsync(h + nr, status, sizeof(int) * nr, cudaMemcpyDeviceToHost, s));
+    LAPH_CUDA(cudaStreamSynchronize(s));
+    InnerStats st;
+    st.iters.assign(h, h + nr);
+    st.status.assign(h + nr, h + 2 * nr);
+    return st;
+}
+
+// BiCGStab in FP64 (the plain solver) on the Schur operator for nr right-hand sides at once, x = 0
+// start, shadow vector r0.  Per-RHS relative stopping on the recursive residual; host polls every
+// `check_every` iterations (device-side scalars, no per-iteration sync).
+static InnerStats bicgstab_schur_f64(laph_ctx *ctx, const DiracOp &op, int nr, const c64 *b, c64 *x, double rel_tol,
+                                     int maxiter, int check_every, cudaStream_t s) {
+    const Geom &g = op.g;
+    long nrows = g.Vh * 12;
+    size_t vb = sizeof(c64) * nrows * nr;
+    auto V = [&](const char *n) { return (c64 *)ws_get(ctx, std::string("in64") + n, vb); };
+    c64 *r = V(":r"), *rh = V(":rh"), *p = V(":p"), *v = V(":v"), *sv = V(":s"), *t = V(":t"), *tmp = V(":tmp");
+    const BicgScalars sc = scalars_get(ctx, "in64:sc", nr);
+    c64 *red = (c64 *)ws_get(ctx, "in64:red", sizeof(c64) * 3 * nr);
     RedPlan pl = red_plan(ctx, nrows, nr);
 
     LAPH_CUDA(cudaMemsetAsync(x, 0, vb, s));
     LAPH_CUDA(cudaMemsetAsync(p, 0, vb, s));
     LAPH_CUDA(cudaMemsetAsync(v, 0, vb, s));
     LAPH_CUDA(cudaMemcpyAsync(r, b, vb, cudaMemcpyDeviceToDevice, s));
-    if constexpr (gen) {
-        mrhs_rhat_init(ctx, pl, nrows, (const c32 *)r, rc, red, s);
-        bicg_init_scalars_gen(nr, sc, red, rel_tol, s);
-    } else {
-        LAPH_CUDA(cudaMemcpyAsync(rh, b, vb, cudaMemcpyDeviceToDevice, s));
-        mrhs_dots<T>(ctx, pl, nrows, 1, r, r, nullptr, nullptr, nullptr, nullptr, red, s);
-        bicg_init_scalars(nr, sc, red, rel_tol, s);
-    }
+    LAPH_CUDA(cudaMemcpyAsync(rh, b, vb, cudaMemcpyDeviceToDevice, s));
+    mrhs_dots<double>(ctx, pl, nrows, 1, r, r, nullptr, nullptr, nullptr, nullptr, red, s);
+    bicg_init_scalars(nr, sc, red, rel_tol, s);
 
-    int *h_flags = (int *)pinned_get(ctx, sizeof(int) * 3 * nr);
     if (check_every < 1) check_every = 5;
     for (int it = 0; it < maxiter; ++it) {
-        bicg_p_update<T>(nrows, nr, sc, r, p, v, s);
-        if constexpr (gen) {   // v = M p with <rhat, v>
-            hop<T>(op, 1, HOP_CLOVINV, tmp, p, nullptr, nullptr, nr, s);
-            if (!hop_f32_xpay_rdot(ctx, op, 0, v, tmp, p, nr, rc, red, s)) {
-                hop<T>(op, 0, HOP_CLOVINV_XPAY, v, tmp, p, nullptr, nr, s);
-                mrhs_rhat_dots(ctx, pl, nrows, v, rc, red, s);
-            }
-        } else {
-            schur_apply<T>(op, nr, p, v, tmp, s);
-            mrhs_dots<T>(ctx, pl, nrows, 1, rh, v, nullptr, nullptr, nullptr, nullptr, red, s);
-        }
+        bicg_p_update<double>(nrows, nr, sc, r, p, v, s);
+        schur_apply<double>(op, nr, p, v, tmp, s);
+        mrhs_dots<double>(ctx, pl, nrows, 1, rh, v, nullptr, nullptr, nullptr, nullptr, red, s);
         bicg_alpha(nr, sc, red, s);
-        bicg_s_update<T>(nrows, nr, sc, r, v, sv, s);
-        schur_apply_tdots<T>(ctx, pl, nrows, op, nr, sv, t, tmp, red, s);
+        bicg_s_update<double>(nrows, nr, sc, r, v, sv, s);
+        schur_apply<double>(op, nr, sv, t, tmp, s);
+        mrhs_dots<double>(ctx, pl, nrows, 2, t, sv, t, t, nullptr, nullptr, red, s);
         bicg_omega(nr, sc, red, s);
-        if constexpr (gen)
-            bicg_xr_update_reduce_gen(ctx, pl, nrows, sc, x, p, sv, t, r, rc, red, s);
-        else
-            bicg_xr_update_reduce<T>(ctx, pl, nrows, sc, x, p, sv, t, r, rh, red, s);
+        bicg_xr_update_reduce<double>(ctx, pl, nrows, sc, x, p, sv, t, r, rh, red, s);
         bicg_rho(nr, sc, red, s);
         if ((it + 1) % check_every == 0 || it + 1 == maxiter) {
+            int *h_flags = (int *)pinned_get(ctx, sizeof(int) * nr);
             LAPH_CUDA(cudaMemcpyAsync(h_flags, sc.active, sizeof(int) * nr, cudaMemcpyDeviceToHost, s));
             LAPH_CUDA(cudaStreamSynchronize(s));
-            hop_timeout_check(s);
             bool any = false;
             for (int k = 0; k < nr; ++k) any |= h_flags[k] != 0;
             if (!any) break;
         }
     }
-    InnerStats st;
-    st.iters.resize(nr);
-    st.status.resize(nr);
-    LAPH_CUDA(cudaMemcpyAsync(h_flags, sc.iters, sizeof(int) * nr, cudaMemcpyDeviceToHost, s));
-    LAPH_CUDA(cudaMemcpyAsync(h_flags + nr, sc.status, sizeof(int) * nr, cudaMemcpyDeviceToHost, s));
-    LAPH_CUDA(cudaStreamSynchronize(s));
-    for (int k = 0; k < nr; ++k) {
-        st.iters[k] = h_flags[k];
-        st.status[k] = h_flags[nr + k];
+    return stats_fetch(ctx, sc.iters, sc.status, nr, s);
+}
+
+// v = M p (or t = M s) with <rhat, v> (K = 1) or the four products of omega and rho (K = 4) as partial sums
+static PartSums schur_apply_sums(laph_ctx *ctx, long nrows, const DiracOp &op, int nr, int K, const c32 *in, c32 *out,
+                                 c32 *tmp, const uint32_t *rc, const int *live, cudaStream_t s) {
+    hop_f32(op, 1, HOP_CLOVINV, tmp, in, nullptr, nr, s, live);
+    PartSums ps;
+    if (K == 1 ? hop_f32_xpay_rdot(ctx, op, 0, out, tmp, in, nr, rc, live, &ps, s)
+               : hop_f32_xpay_dots(ctx, op, 0, out, tmp, in, nr, rc, live, &ps, s))
+        return ps;
+    hop_f32(op, 0, HOP_CLOVINV_XPAY, out, tmp, in, nr, s, live);
+    return bicg32_dots(ctx, nrows, nr, K, live, out, in, rc, s);
+}
+
+// The FP32 inner BiCGStab, streamed: shadow vector the rounded phase of r0 as packed 2-bit codes
+// (blas.cuh), inner products out of the stencil's epilogue where that form exists, updates as in
+// bicg_f32.cu.  Same stopping and polling as the FP64 solver.
+static InnerStats bicgstab_schur_f32(laph_ctx *ctx, const DiracOp &op, int nr, const c32 *b, c32 *x, double rel_tol,
+                                     int maxiter, int check_every, cudaStream_t s) {
+    const long nrows = op.g.Vh * 12;
+    const size_t vb = sizeof(c32) * nrows * nr;
+    auto V = [&](const char *n) { return (c32 *)ws_get(ctx, std::string("in32") + n, vb); };
+    c32 *r = V(":r"), *p = V(":p"), *v = V(":v"), *t = V(":t"), *tmp = V(":tmp");
+    uint32_t *rc = (uint32_t *)ws_get(ctx, "in32:rc", sizeof(uint32_t) * (size_t)(nrows / 12) * nr);
+    const BicgScalars sc = scalars_get(ctx, "in32:sc", nr);
+    c64 *red = (c64 *)ws_get(ctx, "in32:red", sizeof(c64) * 3 * nr);
+    int *live = (int *)ws_get(ctx, "in32:live", sizeof(int));
+    const RedPlan pl = red_plan(ctx, nrows, nr);
+
+    LAPH_CUDA(cudaMemsetAsync(x, 0, vb, s));
+    LAPH_CUDA(cudaMemcpyAsync(r, b, vb, cudaMemcpyDeviceToDevice, s));
+    LAPH_CUDA(cudaMemcpyAsync(p, b, vb, cudaMemcpyDeviceToDevice, s));
+    mrhs_rhat_init(ctx, pl, nrows, r, rc, red, s);
+    bicg_init_scalars_gen(nr, sc, red, rel_tol, s);
+    bicg32_start(nr, sc, live, s);
+
+    if (check_every < 1) check_every = 5;
+    for (int it = 0; it < maxiter; ++it) {
+        const PartSums rv = schur_apply_sums(ctx, nrows, op, nr, 1, p, v, tmp, rc, live, s);   // v = M p
+        bicg32_alpha(ctx, nrows, nr, sc, it == 0, rv, live, s);
+        bicg32_s(ctx, nrows, nr, sc, live, r, v, s);                                           // s, in r
+        const PartSums ts = schur_apply_sums(ctx, nrows, op, nr, 4, r, t, tmp, rc, live, s);   // t = M s
+        bicg32_omega(nr, sc, ts, live, s);
+        bicg32_xrp(ctx, nrows, nr, sc, live, x, r, p, t, v, s);
+        if (it + 1 == maxiter) bicg32_alpha(ctx, nrows, nr, sc, false, PartSums{}, live, s);   // judge the last residual
+        if ((it + 1) % check_every == 0 || it + 1 == maxiter) {
+            int *h = (int *)pinned_get(ctx, sizeof(int));
+            LAPH_CUDA(cudaMemcpyAsync(h, live, sizeof(int), cudaMemcpyDeviceToHost, s));
+            LAPH_CUDA(cudaStreamSynchronize(s));
+            hop_timeout_check(s);
+            if (*h == 0) break;
+        }
     }
-    return st;
+    return stats_fetch(ctx, sc.iters, sc.status, nr, s);
 }
 
 // The FP32 inner solve of a block: in one kernel where the lattice is small, else streamed.
 static InnerStats inner_fp32(laph_ctx *ctx, const DiracOp &op, int nr, const c32 *b, c32 *x, double rel_tol, int maxiter,
                              int check_every, cudaStream_t s) {
-    if (!bicg_small_fits(op, nr)) return bicgstab_schur<float>(ctx, op, nr, b, x, rel_tol, maxiter, check_every, s, "in32");
+    if (!bicg_small_fits(op, nr)) return bicgstab_schur_f32(ctx, op, nr, b, x, rel_tol, maxiter, check_every, s);
     int *d = (int *)ws_get(ctx, "small:stat", sizeof(int) * 2 * nr);
     bicg_small(op, nr, b, x, rel_tol, maxiter, d, d + nr, s);
-    int *h = (int *)pinned_get(ctx, sizeof(int) * 2 * nr);
-    LAPH_CUDA(cudaMemcpyAsync(h, d, sizeof(int) * 2 * nr, cudaMemcpyDeviceToHost, s));
-    LAPH_CUDA(cudaStreamSynchronize(s));
-    InnerStats st;
-    st.iters.assign(h, h + nr);
-    st.status.assign(h + nr, h + 2 * nr);
-    return st;
+    return stats_fetch(ctx, d, d + nr, nr, s);
 }
 
 // The same BiCGStab with every Krylov vector stored in BF16 (one complex per bf2) and FP32
@@ -160,17 +178,7 @@ static InnerStats bicgstab_schur_bf16(laph_ctx *ctx, const DiracOp &op, int nr, 
     size_t vb = sizeof(bf2) * nrows * nr;
     auto V = [&](const char *n) { return (bf2 *)ws_get(ctx, std::string("in16") + n, vb); };
     bf2 *r = V(":r"), *rh = V(":rh"), *p = V(":p"), *v = V(":v"), *sv = V(":s"), *t = V(":t"), *tmp = V(":tmp");
-    char *scb = (char *)ws_get(ctx, "in16:sc", (sizeof(c64) * 4 + sizeof(double) * 2 + sizeof(int) * 3) * nr + 256);
-    BicgScalars sc;
-    sc.rho = (c64 *)scb;
-    sc.alpha = sc.rho + nr;
-    sc.omega = sc.alpha + nr;
-    sc.beta = sc.omega + nr;
-    sc.rr = (double *)(sc.beta + nr);
-    sc.rr_stop = sc.rr + nr;
-    sc.active = (int *)(sc.rr_stop + nr);
-    sc.status = sc.active + nr;
-    sc.iters = sc.status + nr;
+    const BicgScalars sc = scalars_get(ctx, "in16:sc", nr);
     c64 *red = (c64 *)ws_get(ctx, "in16:red", sizeof(c64) * 3 * nr);
     RedPlan pl = red_plan(ctx, nrows, nr);
 
@@ -209,17 +217,7 @@ static InnerStats bicgstab_schur_bf16(laph_ctx *ctx, const DiracOp &op, int nr, 
             if (!any) break;
         }
     }
-    InnerStats st;
-    st.iters.resize(nr);
-    st.status.resize(nr);
-    LAPH_CUDA(cudaMemcpyAsync(h_flags, sc.iters, sizeof(int) * nr, cudaMemcpyDeviceToHost, s));
-    LAPH_CUDA(cudaMemcpyAsync(h_flags + nr, sc.status, sizeof(int) * nr, cudaMemcpyDeviceToHost, s));
-    LAPH_CUDA(cudaStreamSynchronize(s));
-    for (int k = 0; k < nr; ++k) {
-        st.iters[k] = h_flags[k];
-        st.status[k] = h_flags[nr + k];
-    }
-    return st;
+    return stats_fetch(ctx, sc.iters, sc.status, nr, s);
 }
 
 std::vector<int> cgnr_solve(laph_ctx *ctx, const DiracOp &op, int nr, c64 *r, c64 *e,
@@ -364,7 +362,7 @@ void solve_block(laph_ctx *ctx, const DiracOp &op, const c64 *rhs, c64 *sol, int
             // ask the inner solve for what the true residual still needs (Schur and true residuals
             // differ by the clover factor, hence the margin)
             double want = std::max(1e-15, 0.2 * tol / std::max(worst, tol));
-            st = bicgstab_schur<double>(ctx, op, nr, rin, dx, want, budget, prm.check_every, s, "in64");
+            st = bicgstab_schur_f64(ctx, op, nr, rin, dx, want, budget, prm.check_every, s);
             mrhs_axpy_scaled<double, double>(nrows, nr, scale + nr, dx, xe, s);
         } else if (prm.mode == LAPH_SOLVE_MIXED_BF16 && bf16_block_ok(nr)) {
             bf2 *rin = (bf2 *)ws_get(ctx, "dc:rin16", sizeof(bf2) * nrows * nr);
@@ -459,16 +457,18 @@ static int autotune_block(laph_ctx *ctx, const DiracOp &op, int nrhs, cudaStream
     c32 *a = (c32 *)ws_get(ctx, "tune:a", sizeof(c32) * nrows * nmax);
     c32 *b = (c32 *)ws_get(ctx, "tune:b", sizeof(c32) * nrows * nmax);
     c32 *t = (c32 *)ws_get(ctx, "tune:t", sizeof(c32) * nrows * nmax);
-    c64 *red = (c64 *)ws_get(ctx, "tune:red", sizeof(c64) * 2 * nmax);
+    uint32_t *rc = (uint32_t *)ws_get(ctx, "tune:rc", sizeof(uint32_t) * op.g.Vh * nmax);
+    int *live = (int *)ws_get(ctx, "tune:live", sizeof(int));
     LAPH_CUDA(cudaMemsetAsync(a, 0, sizeof(c32) * nrows * nmax, s));
+    LAPH_CUDA(cudaMemsetAsync(rc, 0, sizeof(uint32_t) * op.g.Vh * nmax, s));
+    LAPH_CUDA(cudaMemsetAsync(live, 1, sizeof(int), s));
     cudaEvent_t e0, e1;
     LAPH_CUDA(cudaEventCreate(&e0));
     LAPH_CUDA(cudaEventCreate(&e1));
     int best = cand.back();
     double best_t = 1e300;
     for (int nr : cand) {
-        RedPlan pl = red_plan(ctx, nrows, nr);
-        auto once = [&]() { schur_apply_tdots<float>(ctx, pl, nrows, op, nr, a, b, t, red, s); };
+        auto once = [&]() { (void)schur_apply_sums(ctx, nrows, op, nr, 4, a, b, t, rc, live, s); };
         once();
         LAPH_CUDA(cudaEventRecord(e0, s));
         for (int rep = 0; rep < 3; ++rep) once();
