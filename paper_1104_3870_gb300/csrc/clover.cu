@@ -13,14 +13,16 @@
 // or not finite) raise a flag, and the FP64 kernel does the lattice instead.
 //
 //   1. pack_kernel: coalesced through shared memory; L64, L32w, the limbs by site, the flag.
-//   2. field_kernel: one thread per site and plane; Q - Q^dag from two pairs of leaves that share their
-//      outer link (ten products instead of twelve); F as nine reals by site.
+//   2. field_kernel: one thread per site, plane and pair of leaves that share their outer link (five
+//      products, six leaf by leaf); its part of F as nine reals by site.
 //   3. blocks_kernel: one thread per site and chirality; A and its inverse (L D L^dag in registers),
 //      stored through shared memory in FP64 and in the FP32 form of the stencil.
 // Times at prepare_dirac.
+#include <algorithm>
 #include <cmath>
 
 #include "dirac.cuh"
+#include "fixed.cuh"
 #include "su3.cuh"
 
 namespace laph {
@@ -28,37 +30,8 @@ namespace laph {
 namespace {
 
 // ------------------------------------------------------------------ fixed point
-struct FX {
-    int h, l;
-};
-struct CX {
-    FX re, im;
-};
 struct MX {
     CX m[3][3];
-};
-__device__ __forceinline__ FX neg(FX a) { return {-a.h, -a.l}; }
-
-// round(x 2^58) as limbs, |x| < 2
-__device__ __forceinline__ FX to_fx(double x) {
-    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
-    const int sh = 1027 - (int)((hi >> 20) & 0x7FFu);   // > 63 for zeros and subnormals
-    uint64_t m = (uint64_t)(__funnelshift_l(lo, hi, 11) | 0x80000000u) << 32 | (lo << 11);
-    asm("shr.u64 %0, %0, %1;" : "+l"(m) : "r"(sh));
-    long long f = (long long)((m + 1) >> 1);
-    if (hi >> 31) f = -f;
-    const int h = (int)((f + (1ll << 29)) >> 30);
-    return {h, (int)(f - ((long long)h << 30))};
-}
-// a real of the result: sum of products in units 2^-56
-struct Acc {
-    long long hh = 0, cr = 0;
-    __device__ __forceinline__ void mad(FX a, FX b) {
-        hh += (long long)a.h * b.h;
-        cr += (long long)a.h * b.l;
-        cr += (long long)a.l * b.h;
-    }
-    __device__ __forceinline__ long long value() const { return hh + ((cr + (1ll << 29)) >> 30); }
 };
 __device__ __forceinline__ FX split(long long t) {   // 2^-56 units to limbs
     const int h = (int)((t + (1ll << 27)) >> 28);
@@ -121,8 +94,9 @@ __device__ __forceinline__ int local_site(const Geom &g, long s0, int p, int icb
     return 2 * icb + (c[0] & 1);
 }
 
-__global__ void __launch_bounds__(256) pack_kernel(Geom g, const c64 *__restrict__ U, c64 *__restrict__ L64,
-                                                   float4 *__restrict__ L32w, int4 *__restrict__ fix, int *flag) {
+__global__ void __launch_bounds__(256) pack_kernel(Geom g, const c64 *__restrict__ U, double hws, double hwt,
+                                                   c64 *__restrict__ L64, float4 *__restrict__ L32w,
+                                                   int4 *__restrict__ Lfix, int4 *__restrict__ fix, int *flag) {
     __shared__ double2 sm[PK_SITES * 36];
     __shared__ unsigned char loc[2][PK_SITES / 2];
     const long s0 = (long)blockIdx.x * PK_SITES;
@@ -140,6 +114,9 @@ __global__ void __launch_bounds__(256) pack_kernel(Geom g, const c64 *__restrict
         L64[o] = c64{v.x, v.y};
         const float re = (float)v.x, im = (float)v.y;
         L32w[o] = make_float4(re, re, im, im);
+        const double w = (pm & 3) == 3 ? hwt : hws;
+        const FX a = to_fx(w * v.x), b = to_fx(w * v.y);
+        Lfix[o] = make_int4(a.h, a.l, b.h, b.l);
     }
     for (int e = threadIdx.x; e < 36 * ns; e += 256) {      // [mu][k][site]
         const int is = e % ns, mk = e / ns;
@@ -170,13 +147,15 @@ __device__ __forceinline__ MX load_fix(const int4 *__restrict__ fix, long V, int
     return r;
 }
 
-// F[plane][9][V]: (f00, f11, f22, f10, f20, f21) of the Hermitian traceless F_{mu nu}(x)
+// F[plane][pair][9][V]: the pair's part of (f00, f11, f22, f10, f20, f21) of the Hermitian traceless F_{mu nu}(x).
+// The two pairs run the same code on other links: with both in one thread the code (ten products) missed
+// the instruction cache for a third of the time.
 __global__ void __launch_bounds__(128) field_kernel(Geom g, const int4 *__restrict__ fix, const int *flag,
                                                     double *__restrict__ F) {
     if (*flag) return;
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= g.V) return;
-    const int pl = blockIdx.y;
+    const int pl = blockIdx.y >> 1, pair = blockIdx.y & 1;
     const int mu = pl < 3 ? 0 : pl < 5 ? 1 : 2, nu = pl < 3 ? pl + 1 : pl < 5 ? pl - 1 : 3;
     const int ns = g.ns, nt = g.nt;
     int c[4], r = s;
@@ -192,44 +171,37 @@ __global__ void __launch_bounds__(128) field_kernel(Geom g, const int4 *__restri
     const int nf = c[nu] + 1 == dim[nu] ? -(dim[nu] - 1) * str[nu] : str[nu];
     const int nb = c[nu] == 0 ? (dim[nu] - 1) * str[nu] : -str[nu];
     auto U = [&](int d, int off) { return load_fix(fix, g.V, d, s + off); };
-    // leaf 1 - leaf 4^dag = U_mu(x) { U_nu(x+mu) U_mu(x+nu)^dag U_nu(x)^dag - U_nu(x+mu-nu)^dag U_mu(x-nu)^dag U_nu(x-nu) }
-    MX x = mx_mul<true, true>(U(nu, mf + nb), U(mu, nb));
-    x = mx_mul<false, false>(x, U(nu, nb));
-    MX y = mx_mul<false, true>(U(nu, mf), U(mu, nf));
-    x = mx_mul_sub<false, true>(y, U(nu, 0), x);
-    // leaf 2 - leaf 3^dag = { U_nu(x) U_mu(x-mu+nu)^dag U_nu(x-mu)^dag - U_nu(x-nu)^dag U_mu(x-mu-nu)^dag U_nu(x-mu-nu) } U_mu(x-mu)
-    y = mx_mul<true, true>(U(nu, nb), U(mu, mb + nb));
-    y = mx_mul<false, false>(y, U(nu, mb + nb));
-    MX z = mx_mul<false, true>(U(nu, 0), U(mu, mb + nf));
-    y = mx_mul_sub<false, true>(z, U(nu, mb), y);
-    const MX um = U(mu, 0), ub = U(mu, mb);
+    // pair 0: leaf 1 - leaf 4^dag = U_mu(x) X,
+    //   X = U_nu(x+mu) U_mu(x+nu)^dag U_nu(x)^dag - U_nu(x+mu-nu)^dag U_mu(x-nu)^dag U_nu(x-nu)
+    // pair 1: leaf 2 - leaf 3^dag = X U_mu(x-mu),
+    //   X = U_nu(x) U_mu(x-mu+nu)^dag U_nu(x-mu)^dag - U_nu(x-nu)^dag U_mu(x-mu-nu)^dag U_nu(x-mu-nu)
+    const int a = pair ? 0 : mf, b = pair ? mb : 0;
+    MX x = mx_mul<true, true>(U(nu, a + nb), U(mu, b + nb));
+    x = mx_mul<false, false>(x, U(nu, b + nb));
+    const MX y = mx_mul<false, true>(U(nu, a), U(mu, b + nf));
+    x = mx_mul_sub<false, true>(y, U(nu, b), x);
+    const MX o = U(mu, b), l = pair ? x : o, m = pair ? o : x;
     long long wr[3][3], wi[3][3];
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            long long ar, ai, br, bi;
-            mx_elem<false, false>(um, x, i, j, ar, ai);
-            mx_elem<false, false>(y, ub, i, j, br, bi);
-            wr[i][j] = ar + br;
-            wi[i][j] = ai + bi;
-        }
+        for (int j = 0; j < 3; ++j) mx_elem<false, false>(l, m, i, j, wr[i][j], wi[i][j]);
     // F = (W - W^dag) / (8 i), traceless; W in units 2^-56
     const double u = 1.7347234759768071e-18;   // 2^-59
     double d[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) d[i] = (double)(2 * wi[i][i]) * u;
     const double tr = (double)(2 * (wi[0][0] + wi[1][1] + wi[2][2])) * u * (1.0 / 3.0);
-    double *o = F + (long)pl * 9 * g.V + s;
+    double *f = F + (long)blockIdx.y * 9 * g.V + s;
 #pragma unroll
-    for (int i = 0; i < 3; ++i) o[i * g.V] = d[i] - tr;
+    for (int i = 0; i < 3; ++i) f[i * g.V] = d[i] - tr;
     int k = 3;
 #pragma unroll
     for (int i = 1; i < 3; ++i)
 #pragma unroll
         for (int j = 0; j < i; ++j) {
-            o[k++ * g.V] = (double)(wi[i][j] + wi[j][i]) * u;
-            o[k++ * g.V] = (double)(wr[j][i] - wr[i][j]) * u;
+            f[k++ * g.V] = (double)(wi[i][j] + wi[j][i]) * u;
+            f[k++ * g.V] = (double)(wr[j][i] - wr[i][j]) * u;
         }
 }
 
@@ -351,11 +323,28 @@ __device__ __forceinline__ bool herm6_inverse(Herm6 &a) {
 }
 
 
-// smem [site][2][36] doubles -> FP64 array and FP32 stencil form of the block's sites
+// x 2^n for x of exponent near -n (integer arithmetic; zeros and subnormals give zero)
+__device__ __forceinline__ double scale_pow2(double x, int n) {
+    const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7FF;
+    if (ex == 0 || ex + n <= 0) return 0.0;
+    return __hiloint2double(hi + (n << 20), __double2loint(x));
+}
+
+// smem [site][2][36] doubles -> fixed-point limbs with exponents, FP64 array and FP32 stencil form of the block's sites
 template <int BK_SITES>
-__device__ __forceinline__ void store_blocks(const Geom &g, const double *sm, const unsigned char (*loc)[BK_SITES / 2], long s0,
-                                             int ns, double *__restrict__ a64, float *__restrict__ a32) {
+__device__ __forceinline__ void store_blocks(const Geom &g, const double *sm, const short *ex, const unsigned char (*loc)[BK_SITES / 2], long s0,
+                                             int ns, double *__restrict__ a64, float *__restrict__ a32, int2 *__restrict__ afix,
+                                             int *__restrict__ aexp) {
     const int nh = ns / 2;
+    // limbs of a block's entries over a power of two above them
+    for (int e = threadIdx.x; e < 2 * nh * 72; e += blockDim.x) {
+        const int k = e % 72, icb = (e / 72) % nh, p = e / (72 * nh);
+        const int l = loc[p][icb], E = ex[l * 2 + k / 36];
+        const FX f = to_fx(scale_pow2(sm[l * 73 + k], -E));
+        const long o = (long)p * g.Vh + (s0 >> 1) + icb;
+        afix[o * 72 + k] = make_int2(f.h, f.l);
+        if (k % 36 == 0) aexp[o * 2 + k / 36] = E;
+    }
     for (int e = threadIdx.x; e < 2 * nh * 72; e += blockDim.x) {   // [p][cb][2][36]
         const int k = e % 72, icb = (e / 72) % nh, p = e / (72 * nh);
         a64[((long)p * g.Vh + (s0 >> 1) + icb) * 72 + k] = sm[loc[p][icb] * 73 + k];
@@ -376,8 +365,11 @@ template <int BK_SITES>
 __global__ void __launch_bounds__(2 * BK_SITES) blocks_kernel(Geom g, const double *__restrict__ F, double diag,
                                                               double cs, double ct,
                                                               double *__restrict__ clov64, double *__restrict__ cinv64,
-                                                              float *__restrict__ C32wA, float *__restrict__ C32w) {
+                                                              float *__restrict__ C32wA, float *__restrict__ C32w,
+                                                              int2 *__restrict__ clovfix, int2 *__restrict__ cinvfix,
+                                                              int *__restrict__ clovexp, int *__restrict__ cinvexp) {
     __shared__ double sm[BK_SITES * 73];
+    __shared__ short ex[BK_SITES * 2];     // every entry of the block is below 2^ex
     __shared__ unsigned char loc[2][BK_SITES / 2];
     const long s0 = (long)blockIdx.x * BK_SITES;
     const int ns = (int)min((long)BK_SITES, g.V - s0);
@@ -395,7 +387,10 @@ __global__ void __launch_bounds__(2 * BK_SITES) blocks_kernel(Geom g, const doub
         // G1 = +-c03 F03 - c12 F12, G2 = c02 F02 +- c13 F13, G3 = -c01 F01 +- c23 F23
         auto comb = [&](int pa, double ca, int pb, double cb, double *G) {
 #pragma unroll
-            for (int k = 0; k < 9; ++k) G[k] = fma(cb, __ldg(f + (long)(pb * 9 + k) * g.V), ca * __ldg(f + (long)(pa * 9 + k) * g.V));
+            for (int k = 0; k < 9; ++k) {
+                const double *a = f + (long)(2 * pa * 9 + k) * g.V, *b = f + (long)(2 * pb * 9 + k) * g.V;
+                G[k] = fma(cb, __ldg(b) + __ldg(b + 9 * g.V), ca * (__ldg(a) + __ldg(a + 9 * g.V)));
+            }
         };
         double G1[9], G2[9], G3[9];
         comb(2, sg * ct, 3, -cs, G1);
@@ -429,22 +424,27 @@ __global__ void __launch_bounds__(2 * BK_SITES) blocks_kernel(Geom g, const doub
             o[6 + 2 * i] = a.l[i].re;
             o[6 + 2 * i + 1] = a.l[i].im;
         }
+        uint32_t m = 0;
+#pragma unroll 4
+        for (int i = 0; i < 36; ++i) m = max(m, (uint32_t)__double2hiint(o[i]) & 0x7FFFFFFFu);
+        ex[is * 2 + h] = (short)max((int)(m >> 20) - 1022, -958);
     };
     if (is < ns) put();
     __syncthreads();
-    store_blocks<BK_SITES>(g, sm, loc, s0, ns, clov64, C32wA);
+    store_blocks<BK_SITES>(g, sm, ex, loc, s0, ns, clov64, C32wA, clovfix, clovexp);
     if (is < ns) ok = herm6_inverse(a);
     double piv[36];
     if (!ok) herm6_inverse_pivoted(o, piv);
     __syncthreads();
     if (is < ns) {
-        if (ok)
-            put();
-        else
-            for (int i = 0; i < 36; ++i) o[i] = piv[i];
+        if (!ok) {
+            for (int i = 0; i < 6; ++i) a.d[i] = piv[i];
+            for (int i = 0; i < 15; ++i) a.l[i] = c64{piv[6 + 2 * i], piv[7 + 2 * i]};
+        }
+        put();
     }
     __syncthreads();
-    store_blocks<BK_SITES>(g, sm, loc, s0, ns, cinv64, C32w);
+    store_blocks<BK_SITES>(g, sm, ex, loc, s0, ns, cinv64, C32w, cinvfix, cinvexp);
 }
 
 // ------------------------------------------------------------------ general links (FP64)
@@ -487,7 +487,8 @@ __global__ void __launch_bounds__(64) field_general_kernel(Geom g, const c64 *__
         double d[3];
         for (int i = 0; i < 3; ++i) d[i] = 2.0 * q.m[i][i].im / 8.0;
         const double tr = (d[0] + d[1] + d[2]) / 3.0;
-        double *o = F + (long)pl * 9 * g.V + s;
+        double *o = F + (long)pl * 18 * g.V + s;   // all of it as pair 0
+        for (int k = 9; k < 18; ++k) o[k * g.V] = 0.0;
         for (int i = 0; i < 3; ++i) o[i * g.V] = d[i] - tr;
         int k = 3;
         for (int i = 1; i < 3; ++i)
@@ -501,8 +502,8 @@ __global__ void __launch_bounds__(64) field_general_kernel(Geom g, const c64 *__
 
 }  // namespace
 
-// On 24^3 x 32: pack 0.17, field 2.47, blocks 1.37 ms, 4.0 ms in all; FP64 in one kernel with the blocks
-// in local memory, and four more to convert layouts, took 15.1 ms.  On 16^3 x 32: 1.26 ms (4.6 ms).
+// On 24^3 x 32 3.6 ms in all, for a call of laph_dslash_eo of 4.2 ms; FP64 in one kernel with the blocks
+// in local memory, and four more to convert layouts, took 15.1 of 15.7 ms.
 DiracOp prepare_dirac(laph_ctx *ctx, const Geom &g, const c64 *links, double m0, double csw, double xi, cudaStream_t s) {
     LAPH_REQUIRE(xi > 0.0, "xi must be positive");
     LAPH_REQUIRE(g.V < (1L << 30), "lattice too large for 32-bit site indices");
@@ -519,25 +520,35 @@ DiracOp prepare_dirac(laph_ctx *ctx, const Geom &g, const c64 *links, double m0,
     op.cinv64 = (double *)ws_get(ctx, "dirac:cinv64", sizeof(double) * CLOV_BLOCK * 4 * g.Vh);
     op.C32w = (float *)ws_get(ctx, "dirac:C32w", sizeof(float) * 144 * 2 * g.Vh);
     op.C32wA = (float *)ws_get(ctx, "dirac:C32wA", sizeof(float) * 144 * 2 * g.Vh);
+    op.Lfix = (int4 *)ws_get(ctx, "dirac:Lfix", sizeof(int4) * 9 * 8 * g.Vh);
+    op.clovfix = (int2 *)ws_get(ctx, "dirac:clovfix", sizeof(int2) * CLOV_BLOCK * 4 * g.Vh);
+    op.cinvfix = (int2 *)ws_get(ctx, "dirac:cinvfix", sizeof(int2) * CLOV_BLOCK * 4 * g.Vh);
+    op.clovexp = (int *)ws_get(ctx, "dirac:clovexp", sizeof(int) * 4 * g.Vh);
+    op.cinvexp = (int *)ws_get(ctx, "dirac:cinvexp", sizeof(int) * 4 * g.Vh);
+    op.ctx = ctx;
     int4 *fix = (int4 *)ws_get(ctx, "dirac:fix", sizeof(int4) * 36 * g.V);
-    double *F = (double *)ws_get(ctx, "dirac:F", sizeof(double) * 54 * g.V);
-    int *flag = (int *)ws_get(ctx, "dirac:flag", sizeof(int));
+    double *F = (double *)ws_get(ctx, "dirac:F", sizeof(double) * 108 * g.V);
+    int *flag = (int *)ws_get(ctx, "dirac:flag", 2 * sizeof(int));
+    op.general = flag;
     const double diag = m0 + w[0] + w[1] + w[2] + w[3];
-    LAPH_CUDA(cudaMemsetAsync(flag, 0, sizeof(int), s));
-    pack_kernel<<<grid_for(g.V, PK_SITES), 256, 0, s>>>(g, links, op.L64, op.L32w, fix, flag);
+    LAPH_CUDA(cudaMemsetAsync(flag, 0, 2 * sizeof(int), s));
+    op.weights_bounded = 0.5 * std::max(w[0], w[3]) < 1.0;
+    pack_kernel<<<grid_for(g.V, PK_SITES), 256, 0, s>>>(g, links, op.hw[0], op.hw[3], op.L64, op.L32w, op.Lfix, fix, flag);
     LAPH_LAUNCH_CHECK();
     // small lattices: short blocks, so that the work reaches more SMs
     const bool few = g.V < 32 * 2 * 152;
     const int fb = few ? 32 : 128;
-    field_kernel<<<dim3(grid_for(g.V, fb), 6), fb, 0, s>>>(g, fix, flag, F);
+    field_kernel<<<dim3(grid_for(g.V, fb), 12), fb, 0, s>>>(g, fix, flag, F);
     LAPH_LAUNCH_CHECK();
     field_general_kernel<<<dim3(grid_for(g.V, 64, 512), 6), 64, 0, s>>>(g, links, flag, F);
     LAPH_LAUNCH_CHECK();
     const double cs = -0.5 * csw / xi, ct = -0.25 * csw * (1.0 + 1.0 / xi);
     if (few)
-        blocks_kernel<8><<<grid_for(g.V, 8), 16, 0, s>>>(g, F, diag, cs, ct, op.clov64, op.cinv64, op.C32wA, op.C32w);
+        blocks_kernel<8><<<grid_for(g.V, 8), 16, 0, s>>>(g, F, diag, cs, ct, op.clov64, op.cinv64, op.C32wA, op.C32w,
+                                                            op.clovfix, op.cinvfix, op.clovexp, op.cinvexp);
     else
-        blocks_kernel<32><<<grid_for(g.V, 32), 64, 0, s>>>(g, F, diag, cs, ct, op.clov64, op.cinv64, op.C32wA, op.C32w);
+        blocks_kernel<32><<<grid_for(g.V, 32), 64, 0, s>>>(g, F, diag, cs, ct, op.clov64, op.cinv64, op.C32wA, op.C32w,
+                                                              op.clovfix, op.cinvfix, op.clovexp, op.cinvexp);
     LAPH_LAUNCH_CHECK();
     prepare_f32_operands(ctx, op, s);
     return op;

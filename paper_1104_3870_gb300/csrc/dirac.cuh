@@ -24,6 +24,14 @@ struct DiracOp {
     c64 *L64 = nullptr;      // [2][4][Vh][9]
     double *clov64 = nullptr;  // A       [2][Vh][2][36]
     double *cinv64 = nullptr;  // A^{-1}  [2][Vh][2][36]
+    // fixed-point operands of the FP64 hop (dslash_fix.cu): limbs of hw_mu U, and of the clover blocks
+    // over 2^exp
+    int4 *Lfix = nullptr;     // [2][4][Vh][9] (re.h, re.l, im.h, im.l)
+    int2 *clovfix = nullptr, *cinvfix = nullptr;   // [2][Vh][2][36]
+    int *clovexp = nullptr, *cinvexp = nullptr;    // [2][Vh][2]
+    int *general = nullptr;   // [2] device flags: links not bounded by one; the operand of this hop is not finite
+    bool weights_bounded = true;
+    laph_ctx *ctx = nullptr;  // workspace of the hop's exponents
     // FP32 inner-operator operands in packed form (dslash_f32.cu)
     int *nbr = nullptr;       // [2][Vh][8] neighbour table, sign-folded
     int *order = nullptr;     // [Vh] visiting order of the output sites (z-blocked), see dslash_f32.cu

@@ -128,74 +128,76 @@ struct ClovPtr<double> {
 template <typename T, int MODE>
 __global__ void __launch_bounds__(256) hop_kernel(DiracOp op, int p, cpx<T> *__restrict__ out,
                                                   const cpx<T> *__restrict__ in, const cpx<T> *__restrict__ z,
-                                                  const cpx<T> *__restrict__ xp, int nr) {
+                                                  const cpx<T> *__restrict__ xp, int nr, int behind) {
+    // behind the fixed-point kernel: only what that one left
+    if (behind && !op.general[0] && !op.general[1]) return;
     const Geom &g = op.g;
-    long tid = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    long cb = tid / nr;
-    int r = (int)(tid - cb * nr);
-    if (cb >= g.Vh) return;
-    // neighbours from the table of prepare_f32_operands: forward mu then backward mu, ~j marks
-    // a hop across the time boundary (antiperiodic sign)
-    const int *nb8 = op.nbr + ((long)p * g.Vh + cb) * 8;
-    cpx<T> acc[12];
+    for (long tid = (long)blockIdx.x * blockDim.x + threadIdx.x; tid < g.Vh * nr; tid += (long)gridDim.x * blockDim.x) {
+        long cb = tid / nr;
+        int r = (int)(tid - cb * nr);
+        // neighbours from the table of prepare_f32_operands: forward mu then backward mu, ~j marks
+        // a hop across the time boundary (antiperiodic sign)
+        const int *nb8 = op.nbr + ((long)p * g.Vh + cb) * 8;
+        cpx<T> acc[12];
 #pragma unroll
-    for (int k = 0; k < 12; ++k) acc[k] = {0, 0};
+        for (int k = 0; k < 12; ++k) acc[k] = {0, 0};
 #pragma unroll
-    for (int mu = 0; mu < 4; ++mu) {
-        cpx<T> u[3][3], psi[12];
-        // forward neighbour
-        {
-            int j = __ldg(nb8 + mu);
-            T coef = j < 0 ? -(T)op.hw[mu] : (T)op.hw[mu];
-            long nb = j < 0 ? ~j : j;
-            const cpx<T> *src = in + nb * 12 * nr + r;
+        for (int mu = 0; mu < 4; ++mu) {
+            cpx<T> u[3][3], psi[12];
+            // forward neighbour
+            {
+                int j = __ldg(nb8 + mu);
+                T coef = j < 0 ? -(T)op.hw[mu] : (T)op.hw[mu];
+                long nb = j < 0 ? ~j : j;
+                const cpx<T> *src = in + nb * 12 * nr + r;
 #pragma unroll
-            for (int k = 0; k < 12; ++k) psi[k] = src[(long)k * nr];
-            LinkLoad<T>::load(op, p, mu, cb, u);
-            hop_dir<T>(mu, true, acc, psi, u, coef);
+                for (int k = 0; k < 12; ++k) psi[k] = src[(long)k * nr];
+                LinkLoad<T>::load(op, p, mu, cb, u);
+                hop_dir<T>(mu, true, acc, psi, u, coef);
+            }
+            // backward neighbour
+            {
+                int j = __ldg(nb8 + 4 + mu);
+                T coef = j < 0 ? -(T)op.hw[mu] : (T)op.hw[mu];
+                long nb = j < 0 ? ~j : j;
+                const cpx<T> *src = in + nb * 12 * nr + r;
+#pragma unroll
+                for (int k = 0; k < 12; ++k) psi[k] = src[(long)k * nr];
+                LinkLoad<T>::load(op, 1 - p, mu, nb, u);
+                hop_dir<T>(mu, false, acc, psi, u, coef);
+            }
         }
-        // backward neighbour
-        {
-            int j = __ldg(nb8 + 4 + mu);
-            T coef = j < 0 ? -(T)op.hw[mu] : (T)op.hw[mu];
-            long nb = j < 0 ? ~j : j;
-            const cpx<T> *src = in + nb * 12 * nr + r;
+        cpx<T> res[12];
+        if (MODE == HOP_CLOVINV || MODE == HOP_CLOVINV_XPAY) {
+            const T *ci = ClovPtr<T>::inv(op) + ((long)p * g.Vh + cb) * 2 * CLOV_BLOCK;
+            herm6<T, T>(ci, acc, res);
+            herm6<T, T>(ci + CLOV_BLOCK, acc + 6, res + 6);
+            if (MODE == HOP_CLOVINV_XPAY) {
+                const cpx<T> *zz = z + cb * 12 * nr + r;
 #pragma unroll
-            for (int k = 0; k < 12; ++k) psi[k] = src[(long)k * nr];
-            LinkLoad<T>::load(op, 1 - p, mu, nb, u);
-            hop_dir<T>(mu, false, acc, psi, u, coef);
+                for (int k = 0; k < 12; ++k) res[k] = zz[(long)k * nr] - res[k];
+            }
+        } else {
+            // FP64 only: diagonal A x + hop
+            const double *cl = op.clov64 + ((long)p * g.Vh + cb) * 2 * CLOV_BLOCK;
+            cpx<T> xv[12];
+            const cpx<T> *xx = xp + cb * 12 * nr + r;
+#pragma unroll
+            for (int k = 0; k < 12; ++k) xv[k] = xx[(long)k * nr];
+            herm6<T, double>(cl, xv, res);
+            herm6<T, double>(cl + CLOV_BLOCK, xv + 6, res + 6);
+#pragma unroll
+            for (int k = 0; k < 12; ++k) res[k] += acc[k];
+            if (MODE == HOP_RESID) {
+                const cpx<T> *zz = z + cb * 12 * nr + r;
+#pragma unroll
+                for (int k = 0; k < 12; ++k) res[k] = zz[(long)k * nr] - res[k];
+            }
         }
+        cpx<T> *dst = out + cb * 12 * nr + r;
+#pragma unroll
+        for (int k = 0; k < 12; ++k) dst[(long)k * nr] = res[k];
     }
-    cpx<T> res[12];
-    if (MODE == HOP_CLOVINV || MODE == HOP_CLOVINV_XPAY) {
-        const T *ci = ClovPtr<T>::inv(op) + ((long)p * g.Vh + cb) * 2 * CLOV_BLOCK;
-        herm6<T, T>(ci, acc, res);
-        herm6<T, T>(ci + CLOV_BLOCK, acc + 6, res + 6);
-        if (MODE == HOP_CLOVINV_XPAY) {
-            const cpx<T> *zz = z + cb * 12 * nr + r;
-#pragma unroll
-            for (int k = 0; k < 12; ++k) res[k] = zz[(long)k * nr] - res[k];
-        }
-    } else {
-        // FP64 only: diagonal A x + hop
-        const double *cl = op.clov64 + ((long)p * g.Vh + cb) * 2 * CLOV_BLOCK;
-        cpx<T> xv[12];
-        const cpx<T> *xx = xp + cb * 12 * nr + r;
-#pragma unroll
-        for (int k = 0; k < 12; ++k) xv[k] = xx[(long)k * nr];
-        herm6<T, double>(cl, xv, res);
-        herm6<T, double>(cl + CLOV_BLOCK, xv + 6, res + 6);
-#pragma unroll
-        for (int k = 0; k < 12; ++k) res[k] += acc[k];
-        if (MODE == HOP_RESID) {
-            const cpx<T> *zz = z + cb * 12 * nr + r;
-#pragma unroll
-            for (int k = 0; k < 12; ++k) res[k] = zz[(long)k * nr] - res[k];
-        }
-    }
-    cpx<T> *dst = out + cb * 12 * nr + r;
-#pragma unroll
-    for (int k = 0; k < 12; ++k) dst[(long)k * nr] = res[k];
 }
 
 // Algorithmic traffic of one hop launch over the Vh output sites of a parity:
@@ -215,6 +217,9 @@ double hop_bytes(const DiracOp &op, HopMode mode, int nr, size_t real_bytes) {
 // hopping term) + 504 (two 6x6 complex clover blocks).
 double hop_flops(const DiracOp &op, int nr) { return (double)op.g.Vh * nr * 1824.0; }
 
+bool hop_fix(const DiracOp &op, int p, HopMode mode, c64 *out, const c64 *in, const c64 *z, const c64 *xp, int nr, int block,
+             cudaStream_t s);   // dslash_fix.cu
+
 // Threads per block of a kernel bound by the FP64 pipe of the SMs it runs on: one warp where blocks of
 // four would leave SMs without work (4^3 x 8, 8 right-hand sides: 64 warps, 56 us in blocks of 128).
 static int fp64_block(long n) { return n < 128l * 2 * 152 ? 32 : 128; }
@@ -224,13 +229,14 @@ void hop(const DiracOp &op, int p, HopMode mode, cpx<T> *out, const cpx<T> *in, 
          int nr, cudaStream_t s) {
     long n = op.g.Vh * nr;
     const int block = fp64_block(n);
-    unsigned grid = grid_for(n, block);
     prof_begin("dslash_fp64", s);
+    const int behind = hop_fix(op, p, mode, out, in, z, xp, nr, block, s) ? 1 : 0;
+    const unsigned grid = grid_for(n, block, behind ? 152 * 8 : 1L << 30);
     switch (mode) {
-        case HOP_CLOVINV: hop_kernel<T, HOP_CLOVINV><<<grid, block, 0, s>>>(op, p, out, in, z, xp, nr); break;
-        case HOP_CLOVINV_XPAY: hop_kernel<T, HOP_CLOVINV_XPAY><<<grid, block, 0, s>>>(op, p, out, in, z, xp, nr); break;
-        case HOP_APPLY: hop_kernel<T, HOP_APPLY><<<grid, block, 0, s>>>(op, p, out, in, z, xp, nr); break;
-        case HOP_RESID: hop_kernel<T, HOP_RESID><<<grid, block, 0, s>>>(op, p, out, in, z, xp, nr); break;
+        case HOP_CLOVINV: hop_kernel<T, HOP_CLOVINV><<<grid, block, 0, s>>>(op, p, out, in, z, xp, nr, behind); break;
+        case HOP_CLOVINV_XPAY: hop_kernel<T, HOP_CLOVINV_XPAY><<<grid, block, 0, s>>>(op, p, out, in, z, xp, nr, behind); break;
+        case HOP_APPLY: hop_kernel<T, HOP_APPLY><<<grid, block, 0, s>>>(op, p, out, in, z, xp, nr, behind); break;
+        case HOP_RESID: hop_kernel<T, HOP_RESID><<<grid, block, 0, s>>>(op, p, out, in, z, xp, nr, behind); break;
     }
     LAPH_LAUNCH_CHECK();
     prof_end("dslash_fp64", s, hop_bytes(op, mode, nr, sizeof(T)), hop_flops(op, nr));
