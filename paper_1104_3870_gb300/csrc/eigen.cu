@@ -20,6 +20,7 @@
 #include <cmath>
 #include <vector>
 
+#include "cheb_fix.cuh"
 #include "common.cuh"
 #include "philox.cuh"
 
@@ -514,10 +515,19 @@ struct Lanczos {
     double *nrm, *ca, *cb;
     int *flag;
     int ncheb;
+    ChebFix fix;
+    ChebMap map;
     cudaStream_t s;
     long matvecs = 0;
 
     void apply_A(const c64 *x, c64 *y) {
+        if (fix.usable(map)) {
+            prof_begin("eig_cheb", s);
+            fix.chain(map, ncheb, 1, x, n, y, n, s);
+            prof_end("eig_cheb", s, 0.0, 0.0);
+            matvecs += ncheb;
+            return;
+        }
         // y = T_ncheb(B) x.  T_0 = x (read only); T_k goes to bufs[(ncheb - k) % 3] with
         // bufs = {y, c0, c1}, so T_ncheb lands in y and T_k, T_{k-1}, T_{k-2} never share a buffer.
         long tot = (long)nt * g.V3;
@@ -645,6 +655,9 @@ extern "C" int laph_eigvecs(laph_ctx *ctx, const laph_lattice *lat, const void *
         double *mu = (double *)ws_get(ctx, "eig:mu", sizeof(double) * nt * nv);
         double *res = (double *)ws_get(ctx, "eig:res", sizeof(double) * nt * nv);
         std::vector<double> ha(nt), hb(nt);
+        lz.fix.init(ctx, g, U, s);
+        ChebMap unit;   // -Delta itself
+        unit.set(ctx, "cheb:unit", std::vector<double>(nt, 1.0), std::vector<double>(nt, 0.0), s);
         auto set_map = [&](const std::vector<double> &lamC, int order) {
             for (int t = 0; t < nt; ++t) {
                 if (order == 1 && lamC.empty()) {
@@ -657,6 +670,7 @@ extern "C" int laph_eigvecs(laph_ctx *ctx, const laph_lattice *lat, const void *
             }
             LAPH_CUDA(cudaMemcpyAsync(lz.ca, ha.data(), sizeof(double) * nt, cudaMemcpyHostToDevice, s));
             LAPH_CUDA(cudaMemcpyAsync(lz.cb, hb.data(), sizeof(double) * nt, cudaMemcpyHostToDevice, s));
+            lz.map.set(ctx, "cheb:map", ha, hb, s);
             lz.ncheb = order;
             LAPH_CUDA(cudaStreamSynchronize(s));
         };
@@ -701,14 +715,19 @@ extern "C" int laph_eigvecs(laph_ctx *ctx, const laph_lattice *lat, const void *
             run_jacobi(nt, m, m + 1, lz.H, J, Yraw, Y, theta, false, s);
             rotate(n, nt, m + 1, m, keep, lz.V, Y, Vt, s);
             {
-                std::vector<double> one(nt, 1.0), zero(nt, 0.0);
-                // LY = (-Delta) Y  with a = 1, b = 0 (temporarily swap the map coefficients)
-                LAPH_CUDA(cudaMemcpyAsync(lz.ca, one.data(), sizeof(double) * nt, cudaMemcpyHostToDevice, s));
-                LAPH_CUDA(cudaMemcpyAsync(lz.cb, zero.data(), sizeof(double) * nt, cudaMemcpyHostToDevice, s));
-                long tot = (long)nt * nv * g.V3;
-                cheb_kernel<<<grid_for(tot, 128), 128, 0, s>>>(g, U, nv, Vt, nullptr, LY, lz.ca, lz.cb, 1.0, 0,
-                                                               (long)keep * n, (long)nv * n);
-                LAPH_LAUNCH_CHECK();
+                // LY = (-Delta) Y
+                if (lz.fix.usable(unit)) {
+                    lz.fix.chain(unit, 1, nv, Vt, (long)keep * n, LY, (long)nv * n, s);
+                } else {   // a = 1, b = 0: the map coefficients are swapped for one launch
+                    std::vector<double> one(nt, 1.0), zero(nt, 0.0);
+                    LAPH_CUDA(cudaMemcpyAsync(lz.ca, one.data(), sizeof(double) * nt, cudaMemcpyHostToDevice, s));
+                    LAPH_CUDA(cudaMemcpyAsync(lz.cb, zero.data(), sizeof(double) * nt, cudaMemcpyHostToDevice, s));
+                    long tot = (long)nt * nv * g.V3;
+                    cheb_kernel<<<grid_for(tot, 128), 128, 0, s>>>(g, U, nv, Vt, nullptr, LY, lz.ca, lz.cb, 1.0, 0,
+                                                                   (long)keep * n, (long)nv * n);
+                    LAPH_LAUNCH_CHECK();
+                    LAPH_CUDA(cudaStreamSynchronize(s));
+                }
                 lz.matvecs += nv;
                 ritz_resid_kernel<<<dim3(nv, nt), 256, 0, s>>>(n, nv, keep, nv, Vt, LY, mu, res);
                 LAPH_LAUNCH_CHECK();
@@ -842,12 +861,16 @@ extern "C" int laph_eigvecs(laph_ctx *ctx, const laph_lattice *lat, const void *
                 // filter: T_k into F[(ncheb - k) % 3], T_0 = cur
                 const int npol = ncheb;
                 auto fb = [&](int k) { return F[(npol - k) % 3]; };
-                cheb_kernel<<<cg, 128, 0, s>>>(g, U, keep, cur, nullptr, fb(1), lz.ca, lz.cb, 1.0, 0, ts, ts);
-                LAPH_LAUNCH_CHECK();
-                for (int k = 2; k <= npol; ++k) {
-                    const c64 *tm2 = (k == 2) ? cur : fb(k - 2);
-                    cheb_kernel<<<cg, 128, 0, s>>>(g, U, keep, fb(k - 1), tm2, fb(k), lz.ca, lz.cb, 2.0, 1, ts, ts);
+                if (lz.fix.usable(lz.map)) {
+                    lz.fix.chain(lz.map, npol, keep, cur, ts, F[0], ts, s);
+                } else {
+                    cheb_kernel<<<cg, 128, 0, s>>>(g, U, keep, cur, nullptr, fb(1), lz.ca, lz.cb, 1.0, 0, ts, ts);
                     LAPH_LAUNCH_CHECK();
+                    for (int k = 2; k <= npol; ++k) {
+                        const c64 *tm2 = (k == 2) ? cur : fb(k - 2);
+                        cheb_kernel<<<cg, 128, 0, s>>>(g, U, keep, fb(k - 1), tm2, fb(k), lz.ca, lz.cb, 2.0, 1, ts, ts);
+                        LAPH_LAUNCH_CHECK();
+                    }
                 }
                 lz.matvecs += (long)npol * keep;
                 c64 *Yf = F[0];
@@ -862,8 +885,12 @@ extern "C" int laph_eigvecs(laph_ctx *ctx, const laph_lattice *lat, const void *
                 // Rayleigh-Ritz on -Delta: G = Y^dag L Y, ascending eigenpairs
                 LAPH_CUDA(cudaMemcpyAsync(lz.ca, one.data(), sizeof(double) * nt, cudaMemcpyHostToDevice, s));
                 LAPH_CUDA(cudaMemcpyAsync(lz.cb, zero.data(), sizeof(double) * nt, cudaMemcpyHostToDevice, s));
-                cheb_kernel<<<cg, 128, 0, s>>>(g, U, keep, Yo, nullptr, LK, lz.ca, lz.cb, 1.0, 0, ts, ts);
-                LAPH_LAUNCH_CHECK();
+                if (lz.fix.usable(unit)) {
+                    lz.fix.chain(unit, 1, keep, Yo, ts, LK, ts, s);
+                } else {
+                    cheb_kernel<<<cg, 128, 0, s>>>(g, U, keep, Yo, nullptr, LK, lz.ca, lz.cb, 1.0, 0, ts, ts);
+                    LAPH_LAUNCH_CHECK();
+                }
                 lz.matvecs += keep;
                 gram_kernel<<<gg, 256, 0, s>>>(n, keep, Yo, LK, Gk);
                 LAPH_LAUNCH_CHECK();

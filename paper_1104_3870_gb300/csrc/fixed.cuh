@@ -45,4 +45,32 @@ struct Acc {
     __device__ __forceinline__ long long value() const { return hh + ((cr + (1ll << 29)) >> 30); }
 };
 
+constexpr int EXP_NONE = -2000;   // a spinor of zeros
+constexpr int EXP_MIN = -900;
+
+// floor(x 2^(58 - E)), |x| < 2^E
+__device__ __forceinline__ long long cut(double x, int E) {
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const uint64_t m = fx_shr(fx_mantissa(hi, lo), 1028 + E - (int)((hi >> 20) & 0x7FFu));
+    return (long long)(m ^ (uint64_t)(int64_t)((int32_t)hi >> 31));
+}
+// t 2^-58 as limbs, |t| < 2^59, the low one in [0, 2^30)
+__device__ __forceinline__ FX limbs58(long long t) { return {(int)(t >> 30), (int)((uint32_t)t & 0x3FFFFFFFu)}; }
+// sum of a product in units 2^-56
+__device__ __forceinline__ long long floor_value(const Acc &a) { return a.hh + (a.cr >> 30); }
+__device__ __forceinline__ long long shr_near(long long t, int s) { return s > 0 ? (t + (1ll << (s - 1))) >> s : t; }
+// the double nearest to t 2^q
+__device__ __forceinline__ double to_double(long long t, int q) {
+    if (t == 0) return 0.0;
+    const long long s = t >> 63;
+    const uint64_t a = (uint64_t)((t ^ s) - s);
+    const int lz = __clzll((long long)a);
+    const uint64_t top = a << lz;
+    const uint64_t m = (top >> 11) + ((top >> 10) & 1);   // [2^52, 2^53]
+    const int ex = q + 11 - lz + 1075;
+    if (ex < 1 || ex > 2045) return ldexp((double)t, q);
+    const uint64_t bits = ((uint64_t)ex << 52) + (m - (1ull << 52));
+    return __longlong_as_double((long long)(bits | (uint64_t)s << 63));
+}
+
 }  // namespace laph
