@@ -22,9 +22,12 @@
 
 #include "cheb_fix.cuh"
 #include "common.cuh"
+#include "exact_gemm.cuh"
 #include "philox.cuh"
 
 namespace laph {
+
+void rotate_tc(laph_ctx *ctx, long n, int nt, int ldv, int m, int k, const c64 *V, const c64 *Y, c64 *out, cudaStream_t s);
 
 // Complex Gaussian fill from Philox4x32-10 words by the Box-Muller transform.
 __global__ void normal_fill_kernel(long n, uint32_t seed, uint32_t stream, c64 *out) {
@@ -358,47 +361,6 @@ __global__ void jacobi_kernel(int m, int ldh, const c64 *H, c64 *J, c64 *Y, c64 
     for (int j = threadIdx.x; j < m; j += blockDim.x) theta[(long)t * m + j] = A[(long)order[j] * m + order[j]].re;
 }
 
-// ------------------------------------------------------------------ restart GEMM
-// Out[t][c] = sum_{j < m} V[t][j] Y[t][j][c] for c < k.  Tiled: 64 rows x 16 columns per block.
-__global__ void __launch_bounds__(256) rotate_kernel(long n, int ldv, int m, int k, const c64 *__restrict__ V,
-                                                      const c64 *__restrict__ Y, c64 *__restrict__ Out) {
-    __shared__ c64 Ys[32][16];
-    __shared__ c64 Vs[32][65];
-    int t = blockIdx.z;
-    long r0 = (long)blockIdx.x * 64;
-    int c0 = blockIdx.y * 16;
-    int tr = threadIdx.x % 64, tc = threadIdx.x / 64;   // 64 rows x 4 column groups of 4
-    c64 acc[4] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
-    for (int j0 = 0; j0 < m; j0 += 32) {
-        for (int e = threadIdx.x; e < 32 * 16; e += blockDim.x) {
-            int jj = e / 16, cc = e % 16;
-            int j = j0 + jj, c = c0 + cc;
-            Ys[jj][cc] = (j < m && c < k) ? Y[((long)t * m + j) * m + c] : c64{0, 0};
-        }
-        for (int e = threadIdx.x; e < 32 * 64; e += blockDim.x) {
-            int jj = e / 64, rr = e % 64;
-            int j = j0 + jj;
-            long row = r0 + rr;
-            Vs[jj][rr] = (j < m && row < n) ? V[((long)t * ldv + j) * n + row] : c64{0, 0};
-        }
-        __syncthreads();
-#pragma unroll 4
-        for (int jj = 0; jj < 32; ++jj) {
-            c64 v = Vs[jj][tr];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) acc[q] += v * Ys[jj][tc * 4 + q];
-        }
-        __syncthreads();
-    }
-    long row = r0 + tr;
-    if (row < n)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            int c = c0 + tc * 4 + q;
-            if (c < k) Out[((long)t * k + c) * n + row] = acc[q];
-        }
-}
-
 // ------------------------------------------------------------------ Ritz residuals on -Delta
 // mu[t][i] = <y, L y>, res[t][i] = ||L y - mu y|| for the first nv Ritz vectors (blocks (i, t));
 // Yv holds ldy vectors per slice, LY holds ldl vectors per slice.
@@ -590,12 +552,10 @@ static void run_jacobi(int nt, int m, int ldh, const c64 *H, c64 *J, c64 *Yraw, 
     prof_end("eig_jacobi", s, 0.0, 0.0);
 }
 
-// Out[t][c] = sum_j In[t][j] C[t][j][c]   (k x k coefficients, ldv input vectors per slice)
-static void rotate(long n, int nt, int ldv, int m, int k, const c64 *In, const c64 *C, c64 *Out, cudaStream_t s) {
-    dim3 rg((unsigned)((n + 63) / 64), (unsigned)((k + 15) / 16), nt);
+// Out[t][c] = sum_j In[t][j] C[t][j][c]   (C m x m, of which k columns; ldv input vectors per slice)
+static void rotate(laph_ctx *ctx, long n, int nt, int ldv, int m, int k, const c64 *In, const c64 *C, c64 *Out, cudaStream_t s) {
     prof_begin("eig_gemm", s);
-    rotate_kernel<<<rg, 256, 0, s>>>(n, ldv, m, k, In, C, Out);
-    LAPH_LAUNCH_CHECK();
+    rotate_tc(ctx, n, nt, ldv, m, k, In, C, Out, s);
     prof_end("eig_gemm", s, 0.0, 0.0);
 }
 
@@ -713,7 +673,7 @@ extern "C" int laph_eigvecs(laph_ctx *ctx, const laph_lattice *lat, const void *
         auto cycle = [&](int j0) {
             for (int j = j0; j < m; ++j) lz.step(j);
             run_jacobi(nt, m, m + 1, lz.H, J, Yraw, Y, theta, false, s);
-            rotate(n, nt, m + 1, m, keep, lz.V, Y, Vt, s);
+            rotate(ctx, n, nt, m + 1, m, keep, lz.V, Y, Vt, s);
             {
                 // LY = (-Delta) Y
                 if (lz.fix.usable(unit)) {
@@ -881,7 +841,7 @@ extern "C" int laph_eigvecs(laph_ctx *ctx, const laph_lattice *lat, const void *
                 lowdin_kernel<<<nt, 256, 0, s>>>(keep, Y, theta, Yraw);
                 LAPH_LAUNCH_CHECK();
                 c64 *Yo = (cur == Vt) ? F[1] : Vt;
-                rotate(n, nt, keep, keep, keep, Yf, Yraw, Yo, s);
+                rotate(ctx, n, nt, keep, keep, keep, Yf, Yraw, Yo, s);
                 // Rayleigh-Ritz on -Delta: G = Y^dag L Y, ascending eigenpairs
                 LAPH_CUDA(cudaMemcpyAsync(lz.ca, one.data(), sizeof(double) * nt, cudaMemcpyHostToDevice, s));
                 LAPH_CUDA(cudaMemcpyAsync(lz.cb, zero.data(), sizeof(double) * nt, cudaMemcpyHostToDevice, s));
@@ -896,9 +856,9 @@ extern "C" int laph_eigvecs(laph_ctx *ctx, const laph_lattice *lat, const void *
                 LAPH_LAUNCH_CHECK();
                 run_jacobi(nt, keep, keep, Gk, J, Yraw, Y, theta, true, s);
                 c64 *Yn = (Yo == Vt) ? F[2] : Vt;
-                rotate(n, nt, keep, keep, keep, Yo, Y, Yn, s);
+                rotate(ctx, n, nt, keep, keep, keep, Yo, Y, Yn, s);
                 c64 *LKn = (Yn == F[2]) ? F[0] : F[2];
-                rotate(n, nt, keep, keep, keep, LK, Y, LKn, s);
+                rotate(ctx, n, nt, keep, keep, keep, LK, Y, LKn, s);
                 ritz_resid_kernel<<<dim3(nv, nt), 256, 0, s>>>(n, nv, keep, keep, Yn, LKn, mu, res);
                 LAPH_LAUNCH_CHECK();
                 LAPH_CUDA(cudaMemcpyAsync(lz.ca, ha.data(), sizeof(double) * nt, cudaMemcpyHostToDevice, s));
@@ -945,6 +905,7 @@ extern "C" int laph_eigvecs(laph_ctx *ctx, const laph_lattice *lat, const void *
         LAPH_CUDA(cudaMemcpyAsync(ol.dev, ev.data(), sizeof(double) * ev.size(), cudaMemcpyHostToDevice, s));
         ol.commit(s);
         LAPH_CUDA(cudaStreamSynchronize(s));
+        xg::check_host_flag(ctx);
         if (report) {
             report->restarts = restarts;
             report->matvecs = (int)lz.matvecs;
