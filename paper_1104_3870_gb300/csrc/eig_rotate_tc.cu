@@ -3,7 +3,7 @@
 // Bound by the FP64 pipe in FP64 (four multiply-adds per term at two per cycle and SM); here by the start and
 // drain of short CTAs (m = 80: five sub-chunks) and the partial sums.  The slices go in passes so that those
 // stay below 512 MB.
-// 10^3 x 12, m = 80: about 70 us (1290); N_v = 32 on 16^3 x 32, the whole call, 526 ms (648).
+// 10^3 x 12, m = 56: about 70 us (1290); N_v = 32 on 16^3 x 32, the whole call, 526 ms (648).
 #include "exact_gemm.cuh"
 
 namespace laph {
