@@ -10,7 +10,7 @@
 // applies A to one vector per slice, orthogonalises it against the last two basis
 // vectors and then against the whole basis (full reorthogonalisation) and repeats while the norm drops by more than
 // 1/sqrt(2), at most four repeats.  After m steps the projected matrix is
-// diagonalised (batched complex Jacobi, one block per slice), k Ritz vectors
+// diagonalised (batched complex Jacobi, a cluster per slice), k Ritz vectors
 // are kept (thick restart) and the residuals ||(-Delta) y - mu y|| of the
 // wanted N_v are checked explicitly on -Delta itself.
 //
@@ -224,56 +224,80 @@ __global__ void scale_kernel(long n, c64 *v, const double *nrm) {
 }
 
 // ------------------------------------------------------------------ batched complex Jacobi
-// One block per slice: eigen-decomposition of the Hermitian m x m leading part of H
-// (row stride ldh).  Outputs theta[t][0..m) descending and Y[t][row][col] (eigenvectors in columns).
-__global__ void jacobi_kernel(int m, int ldh, const c64 *H, c64 *J, c64 *Y, c64 *Ysorted, double *theta,
-                              int max_sweeps, int ascending, int in_smem) {
-    extern __shared__ double jsm[];   // reduction scratch, per-pair rotation parameters, [A, Z]
-    const int t = blockIdx.x;
+// Eigen-decomposition of the Hermitian m x m leading part of H (row stride ldh), a cluster of C blocks per
+// slice.  Outputs theta[t][0..m) (descending, or ascending) and Ysorted[t][row][col] (eigenvectors in columns).
+//
+// Bound by the FP64 pipe of the SMs it runs on (two multiply-adds a cycle each), so the work is cut and spread:
+// a round rotates npair disjoint pairs, G^dag A G falls into 2 x 2 blocks (pair k, pair l), and only those with
+// k <= l of the Hermitian A are formed, from the upper triangle of one copy of A in global memory (it stays in
+// L2) into that of the other; the rows of the eigenvector matrix belong to one block each, in shared memory where they
+// fit.  One cluster barrier ends a round.  C is the largest of 8, 4, 2, 1 whose clusters all fit the chip.
+// N_v = 32 on 16^3 x 32 (m = 80, four blocks a slice), the whole call, 321 ms (414 with one block a slice, all of A and Z);
+// m = 56, 12 slices: 3.7 ms a call (8.1).
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ c64 ld_l2(const c64 *p) {
+    const double2 v = __ldcg(reinterpret_cast<const double2 *>(p));
+    return {v.x, v.y};
+}
+__global__ void __launch_bounds__(256) jacobi_kernel(int m, int ldh, const c64 *__restrict__ H, c64 *J, c64 *J2, c64 *Y,
+                                                     c64 *Ysorted, double *theta, int max_sweeps, int ascending, int C,
+                                                     int in_smem) {
+    extern __shared__ double jsm[];   // reduction scratch, per-pair rotation parameters, diagonal, order, [rows of Z]
+    const int t = blockIdx.x / C, rank = blockIdx.x % C;
     const int mm = (m + 1) & ~1;      // even count of players (a dummy index when m is odd)
-    const int npair = mm / 2;
-    double *red = jsm;                 // 2 * blockDim doubles (also the sort order at the end)
-    double *cs = red + 2 * blockDim.x, *sn = cs + npair;
-    c64 *ph = (c64 *)(sn + npair);
-    int *pp = (int *)(ph + npair);
-    int *qq = pp + npair;
-    // the working matrix and the rotations live in shared memory when they fit, else in global
-    c64 *sm_mats = (c64 *)(((uintptr_t)(qq + npair) + 15) & ~(uintptr_t)15);
-    c64 *A = in_smem ? sm_mats : J + (long)t * m * m;
-    c64 *Z = in_smem ? sm_mats + (long)m * m : Y + (long)t * m * m;
+    const int npair = mm / 2, nblk = npair * (npair + 1) / 2;
+    double *red = jsm;                 // 2 * 256
+    double *diag = red + 512;          // mm
+    double *cs = diag + mm, *sn = cs + npair;
+    c64 *ph = (c64 *)(((uintptr_t)(sn + npair) + 15) & ~(uintptr_t)15);
+    int *pp = (int *)(ph + npair), *qq = pp + npair, *order = qq + npair;
+    const int per = (m + C - 1) / C, r0 = min(m, rank * per), nr = min(m, r0 + per) - r0;
+    // Z of row r0 + i and column c at i * zr + c * zc
+    c64 *Z = in_smem ? (c64 *)(((uintptr_t)(order + mm) + 15) & ~(uintptr_t)15) : Y + ((long)t * m + r0) * m;
+    const long zr = in_smem ? 1 : m, zc = in_smem ? nr : 1;
+    c64 *cur = J + (long)t * m * m, *nxt = J2 + (long)t * m * m;
     const c64 *Hs = H + (long)t * ldh * ldh;
-    for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-        int i = e / m, j = e % m;
+    const int gid = rank * 256 + threadIdx.x, gsize = C * 256;
+    for (int e = gid; e < m * m; e += gsize) {
+        const int i = e / m, j = e % m;
+        if (i > j) continue;
         c64 v = 0.5 * (Hs[(long)i * ldh + j] + conj(Hs[(long)j * ldh + i]));
         if (i == j) v.im = 0.0;
-        A[e] = v;
-        Z[e] = c64{i == j ? 1.0 : 0.0, 0.0};
+        cur[e] = v;
     }
-    __syncthreads();
+    for (int e = threadIdx.x; e < nr * m; e += 256) {
+        const int i = e / m, c = e % m;
+        Z[i * zr + c * zc] = c64{r0 + i == c ? 1.0 : 0.0, 0.0};
+    }
+    cluster_barrier();
     for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-        // off-diagonal and total Frobenius norms
+        // off-diagonal and total Frobenius norms, by every block in the same order
         double off = 0.0, tot = 0.0;
-        for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-            double v = norm2(A[e]);
-            tot += v;
-            if (e / m != e % m) off += v;
+        for (int e = threadIdx.x; e < m * m; e += 256) {
+            const int i = e / m, j = e % m;
+            if (i > j) continue;
+            const double v = norm2(ld_l2(cur + e));
+            tot += i == j ? v : 2.0 * v;
+            if (i != j) off += 2.0 * v;
         }
         red[threadIdx.x] = off;
-        red[blockDim.x + threadIdx.x] = tot;
+        red[256 + threadIdx.x] = tot;
         __syncthreads();
-        for (int st = blockDim.x / 2; st > 0; st >>= 1) {
+        for (int st = 128; st > 0; st >>= 1) {
             if ((int)threadIdx.x < st) {
                 red[threadIdx.x] += red[threadIdx.x + st];
-                red[blockDim.x + threadIdx.x] += red[blockDim.x + threadIdx.x + st];
+                red[256 + threadIdx.x] += red[256 + threadIdx.x + st];
             }
             __syncthreads();
         }
-        double offn = red[0], totn = red[blockDim.x];
+        const double offn = red[0], totn = red[256];
         __syncthreads();
         if (offn <= 1e-30 * totn || offn == 0.0) break;
         for (int round = 0; round < mm - 1; ++round) {
             // circle schedule: (mm-1, round) and ((round+k) mod (mm-1), (round-k) mod (mm-1))
-            for (int k = threadIdx.x; k < npair; k += blockDim.x) {
+            for (int k = threadIdx.x; k < npair; k += 256) {
                 int p, q;
                 if (k == 0) {
                     p = mm - 1;
@@ -288,15 +312,18 @@ __global__ void jacobi_kernel(int m, int ldh, const c64 *H, c64 *J, c64 *Y, c64 
                 double c = 1.0, s = 0.0;
                 c64 e{1.0, 0.0};
                 if (q < m) {
-                    c64 apq = A[(long)p * m + q];
-                    double mag = sqrt(norm2(apq));
+                    const c64 apq = ld_l2(cur + (long)p * m + q);
+                    const double app = ld_l2(cur + (long)p * m + p).re, aqq = ld_l2(cur + (long)q * m + q).re;
+                    const double mag = sqrt(norm2(apq));
                     if (mag > 1e-300) {
-                        double app = A[(long)p * m + p].re, aqq = A[(long)q * m + q].re;
-                        double tau = (aqq - app) / (2.0 * mag);
-                        double tt = (tau >= 0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-                        c = 1.0 / sqrt(1.0 + tt * tt);
-                        s = -tt * c;   // G = diag(1, e^{-i phi}) [[c, -s], [s, c]] zeroes A_pq
-                        e = c64{apq.re / mag, apq.im / mag};   // e^{i phi}
+                        const double tau = (aqq - app) / (2.0 * mag);
+                        const double tt = (tau >= 0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
+                        const double ct = 1.0 / sqrt(1.0 + tt * tt), st = -tt * ct;
+                        if (st != 0.0) {   // G = diag(1, e^{-i phi}) [[c, -s], [s, c]] zeroes A_pq
+                            c = ct;
+                            s = st;
+                            e = c64{apq.re / mag, apq.im / mag};   // e^{i phi}
+                        }
                     }
                 }
                 cs[k] = c;
@@ -304,61 +331,84 @@ __global__ void jacobi_kernel(int m, int ldh, const c64 *H, c64 *J, c64 *Y, c64 
                 ph[k] = e;
             }
             __syncthreads();
-            // rows: A <- G^dag A, G = [[c, -s], [s e^{-i phi}, c e^{-i phi}]] on (p, q)
-            for (int e2 = threadIdx.x; e2 < npair * m; e2 += blockDim.x) {
-                int k = e2 / m, j = e2 % m;
-                int p = pp[k], q = qq[k];
-                if (q >= m || sn[k] == 0.0) continue;
-                c64 ep = ph[k];
-                c64 apj = A[(long)p * m + j], aqj = A[(long)q * m + j];
-                A[(long)p * m + j] = cs[k] * apj + sn[k] * (ep * aqj);
-                A[(long)q * m + j] = (-sn[k]) * apj + cs[k] * (ep * aqj);
+            for (int b = gid; b < nblk; b += gsize) {
+                int l = (int)((sqrtf(8.0f * b + 1.0f) - 1.0f) * 0.5f);
+                while ((l + 1) * (l + 2) / 2 <= b) ++l;
+                while (l * (l + 1) / 2 > b) --l;
+                const int k = b - l * (l + 1) / 2;   // k <= l
+                const int ra[2] = {pp[k], qq[k]}, cb[2] = {pp[l], qq[l]};
+                c64 M[2][2];
+#pragma unroll
+                for (int u = 0; u < 2; ++u)
+#pragma unroll
+                    for (int v = 0; v < 2; ++v) {
+                        const int i = ra[u], j = cb[v];
+                        M[u][v] = c64{0, 0};
+                        if (i < m && j < m) {
+                            const c64 z = ld_l2(cur + (i <= j ? (long)i * m + j : (long)j * m + i));
+                            M[u][v] = i <= j ? z : conj(z);
+                        }
+                    }
+                const double ck = cs[k], sk = sn[k], cl = cs[l], sl = sn[l];
+                const c64 ek = ph[k], el = conj(ph[l]);
+#pragma unroll
+                for (int v = 0; v < 2; ++v) {   // G^dag A: G = [[c, -s], [s e^{-i phi}, c e^{-i phi}]] on (p, q)
+                    const c64 x = M[0][v], y = ek * M[1][v];
+                    M[0][v] = ck * x + sk * y;
+                    M[1][v] = (-sk) * x + ck * y;
+                }
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const c64 x = M[u][0], y = M[u][1] * el;
+                    M[u][0] = cl * x + sl * y;
+                    M[u][1] = (-sl) * x + cl * y;
+                }
+                if (k == l) {
+                    M[0][0].im = M[1][1].im = 0.0;
+                    if (sk != 0.0) M[0][1] = c64{0, 0};
+                }
+#pragma unroll
+                for (int u = 0; u < 2; ++u)
+#pragma unroll
+                    for (int v = 0; v < 2; ++v) {
+                        const int i = ra[u], j = cb[v];
+                        if (i >= m || j >= m || (k == l && u > v)) continue;
+                        nxt[i <= j ? (long)i * m + j : (long)j * m + i] = i <= j ? M[u][v] : conj(M[u][v]);
+                    }
             }
-            __syncthreads();
-            // columns: A <- A G,  Z <- Z G
-            for (int e2 = threadIdx.x; e2 < npair * m; e2 += blockDim.x) {
-                int k = e2 / m, i = e2 % m;
-                int p = pp[k], q = qq[k];
-                if (q >= m || sn[k] == 0.0) continue;
-                c64 em = conj(ph[k]);
-                c64 aip = A[(long)i * m + p], aiq = A[(long)i * m + q];
-                A[(long)i * m + p] = cs[k] * aip + sn[k] * (aiq * em);
-                A[(long)i * m + q] = (-sn[k]) * aip + cs[k] * (aiq * em);
-                c64 zip = Z[(long)i * m + p], ziq = Z[(long)i * m + q];
-                Z[(long)i * m + p] = cs[k] * zip + sn[k] * (ziq * em);
-                Z[(long)i * m + q] = (-sn[k]) * zip + cs[k] * (ziq * em);
+            // Z <- Z G on this block's rows
+            for (int e2 = threadIdx.x; e2 < npair * nr; e2 += 256) {
+                const int k = e2 / nr, i = e2 % nr, p = pp[k], q = qq[k];
+                const double c = cs[k], s = sn[k];
+                if (q >= m || s == 0.0) continue;
+                c64 *zp = Z + i * zr + p * zc, *zq = Z + i * zr + q * zc;
+                const c64 x = *zp, y = *zq * conj(ph[k]);
+                *zp = c * x + s * y;
+                *zq = (-s) * x + c * y;
             }
-            __syncthreads();
-            for (int k = threadIdx.x; k < npair; k += blockDim.x) {
-                int p = pp[k], q = qq[k];
-                if (q >= m || sn[k] == 0.0) continue;
-                A[(long)p * m + q] = c64{0, 0};
-                A[(long)q * m + p] = c64{0, 0};
-                A[(long)p * m + p].im = 0.0;
-                A[(long)q * m + q].im = 0.0;
-            }
-            __syncthreads();
+            cluster_barrier();
+            c64 *tmp = cur;
+            cur = nxt;
+            nxt = tmp;
         }
     }
-    // sort descending (thread 0 builds the order, all threads permute)
-    int *order = (int *)red;
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < m; ++i) order[i] = i;
+    for (int j = threadIdx.x; j < m; j += 256) diag[j] = ld_l2(cur + (long)j * m + j).re;
+    __syncthreads();
+    for (int j = threadIdx.x; j < m; j += 256) {
+        const double v = diag[j];
+        int pos = 0;
         for (int i = 0; i < m; ++i) {
-            int best = i;
-            for (int j = i + 1; j < m; ++j) {
-                double vj = A[(long)order[j] * m + order[j]].re, vb = A[(long)order[best] * m + order[best]].re;
-                if (ascending ? vj < vb : vj > vb) best = j;
-            }
-            int tmp = order[i]; order[i] = order[best]; order[best] = tmp;
+            const double o = diag[i];
+            pos += (ascending ? o < v : o > v) || (o == v && i < j) || (v != v && (o == o || i < j));
         }
+        order[min(pos, m - 1)] = j;
+        if (rank == 0) theta[(long)t * m + min(pos, m - 1)] = v;
     }
     __syncthreads();
-    for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-        int i = e / m, j = e % m;
-        Ysorted[(long)t * m * m + e] = Z[(long)i * m + order[j]];
+    for (int e = threadIdx.x; e < nr * m; e += 256) {
+        const int i = e / m, j = e % m;
+        Ysorted[((long)t * m + r0 + i) * m + j] = Z[i * zr + order[j] * zc];
     }
-    for (int j = threadIdx.x; j < m; j += blockDim.x) theta[(long)t * m + j] = A[(long)order[j] * m + order[j]].re;
 }
 
 // ------------------------------------------------------------------ Ritz residuals on -Delta
@@ -543,20 +593,35 @@ struct Lanczos {
 };
 
 // Eigen-decomposition of the leading m x m Hermitian part of H[t] (row stride ldh) for every slice.
-static void run_jacobi(int nt, int m, int ldh, const c64 *H, c64 *J, c64 *Yraw, c64 *Y, double *theta, bool ascending,
-                       cudaStream_t s) {
-    int npair = ((m + 1) & ~1) / 2;
+static void run_jacobi(laph_ctx *ctx, int nt, int m, int ldh, const c64 *H, c64 *J, c64 *Yraw, c64 *Y, double *theta,
+                       bool ascending, cudaStream_t s) {
+    const int mm = (m + 1) & ~1, npair = mm / 2;
     LAPH_REQUIRE(m <= 1024, "Krylov dimension above 1024 is not supported");
-    size_t shm = sizeof(double) * 2 * 256 + sizeof(double) * 2 * npair + sizeof(c64) * npair + sizeof(int) * 2 * npair;
-    size_t mats = 2 * sizeof(c64) * (size_t)m * m + 16;
-    const size_t smem_cap = 220 * 1024;   // below the 227 KB opt-in limit per block
-    int in_smem = (shm + mats <= smem_cap) ? 1 : 0;
+    c64 *J2 = (c64 *)ws_get(ctx, "eig:J2", sizeof(c64) * nt * (size_t)m * m);
+    const int sms = ctx->sm_count > 0 ? ctx->sm_count : 152;
+    int C = 8;
+    while (C > 1 && (long)C * nt > sms) C /= 2;
+    const int per = (m + C - 1) / C;
+    size_t shm = sizeof(double) * (512 + mm + 2 * npair) + 16 + sizeof(c64) * npair + sizeof(int) * (2 * npair + mm) + 16;
+    const size_t rows = sizeof(c64) * (size_t)per * m;
+    const int in_smem = shm + rows <= 220 * 1024 ? 1 : 0;   // below the 227 KB opt-in limit per block
     if (in_smem) {
-        shm += mats;
+        shm += rows;
         LAPH_CUDA(cudaFuncSetAttribute(jacobi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
     }
     prof_begin("eig_jacobi", s);
-    jacobi_kernel<<<nt, 256, shm, s>>>(m, ldh, H, J, Yraw, Y, theta, 60, ascending ? 1 : 0, in_smem);
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)C;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)(nt * C));
+    cfg.blockDim = dim3(256);
+    cfg.dynamicSmemBytes = shm;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    LAPH_CUDA(cudaLaunchKernelEx(&cfg, jacobi_kernel, m, ldh, H, J, J2, Yraw, Y, theta, 60, ascending ? 1 : 0, C, in_smem));
     LAPH_LAUNCH_CHECK();
     prof_end("eig_jacobi", s, 0.0, 0.0);
 }
@@ -668,7 +733,7 @@ extern "C" int laph_eigvecs(laph_ctx *ctx, const laph_lattice *lat, const void *
             start_vector();
             int mest = std::min(m, nv + 24);   // enough Ritz values to bound lambda_{nv+8} from above
             for (int j = 0; j < mest; ++j) lz.step(j);
-            run_jacobi(nt, mest, m + 1, lz.H, J, Yraw, Y, theta, false, s);
+            run_jacobi(ctx, nt, mest, m + 1, lz.H, J, Yraw, Y, theta, false, s);
             LAPH_CUDA(cudaMemcpyAsync(h_theta.data(), theta, sizeof(double) * nt * mest, cudaMemcpyDeviceToHost, s));
             LAPH_CUDA(cudaStreamSynchronize(s));
             int idx = std::min(nv + 8, mest - 1);
@@ -681,7 +746,7 @@ extern "C" int laph_eigvecs(laph_ctx *ctx, const laph_lattice *lat, const void *
         // and the Rayleigh quotients mu and residuals of the nv wanted ones on -Delta itself.
         auto cycle = [&](int j0) {
             for (int j = j0; j < m; ++j) lz.step(j);
-            run_jacobi(nt, m, m + 1, lz.H, J, Yraw, Y, theta, false, s);
+            run_jacobi(ctx, nt, m, m + 1, lz.H, J, Yraw, Y, theta, false, s);
             rotate(ctx, n, nt, m + 1, m, keep, lz.V, Y, Vt, s);
             {
                 // LY = (-Delta) Y
@@ -846,7 +911,7 @@ extern "C" int laph_eigvecs(laph_ctx *ctx, const laph_lattice *lat, const void *
                 // Loewdin: S = Yf^dag Yf = W diag(w) W^dag, Y = Yf W diag(w)^{-1/2}
                 gram_kernel<<<gg, 256, 0, s>>>(n, keep, Yf, Yf, Gk);
                 LAPH_LAUNCH_CHECK();
-                run_jacobi(nt, keep, keep, Gk, J, Yraw, Y, theta, false, s);
+                run_jacobi(ctx, nt, keep, keep, Gk, J, Yraw, Y, theta, false, s);
                 lowdin_kernel<<<nt, 256, 0, s>>>(keep, Y, theta, Yraw);
                 LAPH_LAUNCH_CHECK();
                 c64 *Yo = (cur == Vt) ? F[1] : Vt;
@@ -863,7 +928,7 @@ extern "C" int laph_eigvecs(laph_ctx *ctx, const laph_lattice *lat, const void *
                 lz.matvecs += keep;
                 gram_kernel<<<gg, 256, 0, s>>>(n, keep, Yo, LK, Gk);
                 LAPH_LAUNCH_CHECK();
-                run_jacobi(nt, keep, keep, Gk, J, Yraw, Y, theta, true, s);
+                run_jacobi(ctx, nt, keep, keep, Gk, J, Yraw, Y, theta, true, s);
                 c64 *Yn = (Yo == Vt) ? F[2] : Vt;
                 rotate(ctx, n, nt, keep, keep, keep, Yo, Y, Yn, s);
                 c64 *LKn = (Yn == F[2]) ? F[0] : F[2];
