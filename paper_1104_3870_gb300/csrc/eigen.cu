@@ -144,13 +144,12 @@ __device__ __forceinline__ c64 block_sum(c64 v, c64 *sm) {
     return r;
 }
 
-// h[t][i] = <V[t][i], w[t]> for i < cnt; blocks (t, i); skipped for slices whose flag is 0 when pass > 0
+// h[t][i] = <V[t][i], w[t]> for i < cnt; blocks (t, i)
 __global__ void gemv_c_kernel(long n, int ldv, const c64 *__restrict__ V, const c64 *__restrict__ w, int cnt,
-                              c64 *h, const int *flag, int pass) {
+                              c64 *h) {
     __shared__ c64 sm[256];
     int t = blockIdx.y, i = blockIdx.x;
     if (i >= cnt) return;
-    if (pass > 0 && !flag[t]) return;
     const c64 *v = V + ((long)t * ldv + i) * n;
     const c64 *ww = w + (long)t * n;
     c64 a{0, 0};
@@ -159,11 +158,9 @@ __global__ void gemv_c_kernel(long n, int ldv, const c64 *__restrict__ V, const 
     if (threadIdx.x == 0) h[(long)t * (ldv + 1) + i] = s;
 }
 
-// w[t] -= sum_i V[t][i] h[t][i];  hacc += h
-__global__ void gemv_n_kernel(long n, int ldv, const c64 *__restrict__ V, c64 *w, int cnt, const c64 *__restrict__ h,
-                              const int *flag, int pass) {
+// w[t] -= sum_i V[t][i] h[t][i]
+__global__ void gemv_n_kernel(long n, int ldv, const c64 *__restrict__ V, c64 *w, int cnt, const c64 *__restrict__ h) {
     int t = blockIdx.y;
-    if (pass > 0 && !flag[t]) return;
     long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
     const c64 *hh = h + (long)t * (ldv + 1);
@@ -172,14 +169,12 @@ __global__ void gemv_n_kernel(long n, int ldv, const c64 *__restrict__ V, c64 *w
     w[(long)t * n + k] -= s;
 }
 
-// nrm[t] = ||w[t]||; flag[t] = another pass needed (norm fell by more than 1/sqrt 2, < 4 repeats);
-// accumulates h into column j of H (pass > 0 only for flagged slices).
+// nrm[t] = ||w[t]||; flag[t] = another pass needed (norm fell by more than 1/sqrt 2); accumulates h into
+// column j of H.
 __global__ void reorth_norm_kernel(long n, int ldv, const c64 *w, const c64 *h, c64 *H, int j, int cnt, double *nrm,
-                                   int *flag, int pass) {
+                                   int *flag) {
     __shared__ c64 sm[256];
     int t = blockIdx.x;
-    bool active = pass == 0 || flag[t];
-    if (!active) return;
     const c64 *ww = w + (long)t * n;
     c64 a{0, 0};
     for (long k = threadIdx.x; k < n; k += blockDim.x) a += c64{norm2(ww[k]), 0.0};
@@ -191,7 +186,7 @@ __global__ void reorth_norm_kernel(long n, int ldv, const c64 *w, const c64 *h, 
         double after = sqrt(s.re);
         double before = nrm[t];
         nrm[t] = after;
-        flag[t] = (pass < 4 && after < before * 0.7071067811865476) ? 1 : 0;
+        flag[t] = after < before * 0.7071067811865476 ? 1 : 0;
     }
 }
 
@@ -203,6 +198,82 @@ __global__ void norm_only_kernel(long n, const c64 *w, double *nrm) {
     for (long k = threadIdx.x; k < n; k += blockDim.x) a += c64{norm2(ww[k]), 0.0};
     c64 s = block_sum(a, sm);
     if (threadIdx.x == 0) nrm[t] = sqrt(s.re);
+}
+
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ c64 ld_l2(const c64 *p) {
+    const double2 v = __ldcg(reinterpret_cast<const double2 *>(p));
+    return {v.x, v.y};
+}
+
+// The end of a Lanczos step, a cluster of STEP_C blocks per slice, each with a range of the vector: the further
+// passes of the orthogonalisation for the slices whose flag asks for them (at most four), then V[j+1] = w / nrm, the
+// same into next (the operand of the next step) and H[j+1][j] = nrm.  Most steps need no further pass: as separate
+// launches the four passes, the scaling and the copy were fourteen nearly empty kernels, 40 us a step.
+// 6^3 x 8, N_v = 12, the whole call 25.3 ms (30.3); 16^3 x 32, N_v = 32: 305 ms (321).
+constexpr int STEP_C = 8;
+__global__ void __launch_bounds__(256) lanczos_end_kernel(long n, int ldv, int j, c64 *V, c64 *w, c64 *part, c64 *H, double *nrm,
+                                                          int *flag, c64 *next) {
+    extern __shared__ c64 esm[];   // h of this pass [j + 1]
+    __shared__ double red[8];
+    const int t = blockIdx.x / STEP_C, rank = blockIdx.x % STEP_C, cnt = j + 1;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const long per = (n + STEP_C - 1) / STEP_C, k0 = min(n, rank * per), k1 = min(n, k0 + per);
+    c64 *Vt = V + (long)t * ldv * n, *ww = w + (long)t * n, *Ht = H + (long)t * ldv * ldv;
+    c64 *pt = part + (long)t * STEP_C * (ldv + 1);   // [rank][ldv + 1], the last for the norm
+    double b = nrm[t];
+    bool again = flag[t] != 0;
+    for (int pass = 1; pass <= 4 && again; ++pass) {
+        for (int i = warp; i < cnt; i += 8) {
+            c64 a{0, 0};
+            for (long k = k0 + lane; k < k1; k += 32) a += cmul_conj(Vt[(long)i * n + k], ww[k]);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                a.re += __shfl_xor_sync(0xffffffffu, a.re, o);
+                a.im += __shfl_xor_sync(0xffffffffu, a.im, o);
+            }
+            if (lane == 0) pt[(long)rank * (ldv + 1) + i] = a;
+        }
+        cluster_barrier();
+        for (int i = threadIdx.x; i < cnt; i += 256) {
+            c64 a{0, 0};
+            for (int r = 0; r < STEP_C; ++r) a += ld_l2(pt + (long)r * (ldv + 1) + i);
+            esm[i] = a;
+            if (rank == 0) Ht[(long)i * ldv + j] += a;
+        }
+        __syncthreads();
+        double q = 0.0;
+        for (long k = k0 + threadIdx.x; k < k1; k += 256) {
+            c64 a{0, 0};
+            for (int i = 0; i < cnt; ++i) a += Vt[(long)i * n + k] * esm[i];
+            a = ww[k] - a;
+            ww[k] = a;
+            q += norm2(a);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+        if (lane == 0) red[warp] = q;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int i = 1; i < 8; ++i) q += red[i];
+            pt[(long)rank * (ldv + 1) + ldv] = c64{q, 0.0};
+        }
+        cluster_barrier();
+        double after = 0.0;
+        for (int r = 0; r < STEP_C; ++r) after += ld_l2(pt + (long)r * (ldv + 1) + ldv).re;
+        after = sqrt(after);
+        again = pass < 4 && after < b * 0.7071067811865476;
+        b = after;
+    }
+    const double inv = b > 0.0 ? 1.0 / b : 0.0;
+    for (long k = k0 + threadIdx.x; k < k1; k += 256) {
+        const c64 v = inv * ww[k];
+        Vt[(long)(j + 1) * n + k] = v;
+        next[(long)t * n + k] = v;
+    }
+    if (rank == 0 && threadIdx.x == 0 && j + 1 < ldv) Ht[(long)(j + 1) * ldv + j] = c64{b, 0.0};
 }
 
 // V[t][j+1] = w / nrm; H[j+1][j] = nrm (when j+1 < ldv rows)
@@ -234,13 +305,6 @@ __global__ void scale_kernel(long n, c64 *v, const double *nrm) {
 // fit.  One cluster barrier ends a round.  C is the largest of 8, 4, 2, 1 whose clusters all fit the chip.
 // N_v = 32 on 16^3 x 32 (m = 80, four blocks a slice), the whole call, 321 ms (414 with one block a slice, all of A and Z);
 // m = 56, 12 slices: 3.7 ms a call (8.1).
-__device__ __forceinline__ void cluster_barrier() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ c64 ld_l2(const c64 *p) {
-    const double2 v = __ldcg(reinterpret_cast<const double2 *>(p));
-    return {v.x, v.y};
-}
 __global__ void __launch_bounds__(256) jacobi_kernel(int m, int ldh, const c64 *__restrict__ H, c64 *J, c64 *J2, c64 *Y,
                                                      c64 *Ysorted, double *theta, int max_sweeps, int ascending, int C,
                                                      int in_smem) {
@@ -523,7 +587,7 @@ struct Lanczos {
     long n;
     int nt, m, ldv;   // ldv = m + 1 basis vectors
     const c64 *U;
-    c64 *V, *w, *c0, *c1, *H, *h;
+    c64 *V, *w, *c0, *c1, *H, *h, *part;
     double *nrm, *ca, *cb;
     int *flag;
     int ncheb;
@@ -560,9 +624,13 @@ struct Lanczos {
 
     // One Lanczos step j: V[:, j+1] from A V[:, j], full reorthogonalisation.
     void step(int j) {
-        // w = A v_j; v_j (slice t at V + (t*ldv + j)*n) is first gathered into a dense [t][n] block
-        copy_slices_kernel<<<dim3(grid_for(n, 256), nt), 256, 0, s>>>(n, V + (long)j * n, (long)ldv * n, h_vec, n);
-        LAPH_LAUNCH_CHECK();
+        // w = A v_j; v_j (slice t at V + (t*ldv + j)*n) as a dense [t][n] block: left by the step before, gathered
+        // behind a start vector or a restart
+        if (!have_vec) {
+            copy_slices_kernel<<<dim3(grid_for(n, 256), nt), 256, 0, s>>>(n, V + (long)j * n, (long)ldv * n, h_vec, n);
+            LAPH_LAUNCH_CHECK();
+        }
+        have_vec = true;
         apply_A(h_vec, w);
         int cnt = j + 1;
         prof_begin("eig_reorth", s);
@@ -571,25 +639,35 @@ struct Lanczos {
         // longer falls; the flags still call for more where it does, as behind a restart).  The passes are
         // bound by the FP64 pipe and by reading V; N_v = 32 on 16^3 x 32, the whole call, 414 ms (526).
         const int l0 = std::max(j - 1, 0), lc = cnt - l0;
-        gemv_c_kernel<<<dim3(lc, nt), 256, 0, s>>>(n, ldv, V + (long)l0 * n, w, lc, h, flag, 0);
+        gemv_c_kernel<<<dim3(lc, nt), 256, 0, s>>>(n, ldv, V + (long)l0 * n, w, lc, h);
         LAPH_LAUNCH_CHECK();
-        gemv_n_kernel<<<dim3(grid_for(n, 256), nt), 256, 0, s>>>(n, ldv, V + (long)l0 * n, w, lc, h, flag, 0);
+        gemv_n_kernel<<<dim3(grid_for(n, 256), nt), 256, 0, s>>>(n, ldv, V + (long)l0 * n, w, lc, h);
         LAPH_LAUNCH_CHECK();
-        reorth_norm_kernel<<<nt, 256, 0, s>>>(n, ldv, w, h, H + (long)l0 * ldv, j, lc, nrm, flag, 0);
+        reorth_norm_kernel<<<nt, 256, 0, s>>>(n, ldv, w, h, H + (long)l0 * ldv, j, lc, nrm, flag);
         LAPH_LAUNCH_CHECK();
-        for (int pass = 0; pass <= 4; ++pass) {
-            gemv_c_kernel<<<dim3(cnt, nt), 256, 0, s>>>(n, ldv, V, w, cnt, h, flag, pass);
-            LAPH_LAUNCH_CHECK();
-            gemv_n_kernel<<<dim3(grid_for(n, 256), nt), 256, 0, s>>>(n, ldv, V, w, cnt, h, flag, pass);
-            LAPH_LAUNCH_CHECK();
-            reorth_norm_kernel<<<nt, 256, 0, s>>>(n, ldv, w, h, H, j, cnt, nrm, flag, pass);
-            LAPH_LAUNCH_CHECK();
-        }
+        gemv_c_kernel<<<dim3(cnt, nt), 256, 0, s>>>(n, ldv, V, w, cnt, h);
+        LAPH_LAUNCH_CHECK();
+        gemv_n_kernel<<<dim3(grid_for(n, 256), nt), 256, 0, s>>>(n, ldv, V, w, cnt, h);
+        LAPH_LAUNCH_CHECK();
+        reorth_norm_kernel<<<nt, 256, 0, s>>>(n, ldv, w, h, H, j, cnt, nrm, flag);
+        LAPH_LAUNCH_CHECK();
         prof_end("eig_reorth", s, 0.0, 0.0);
-        lanczos_next_kernel<<<dim3(grid_for(n, 256), nt), 256, 0, s>>>(n, ldv, j, w, nrm, V, H);
+        cudaLaunchConfig_t cfg{};
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = STEP_C;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cfg.gridDim = dim3((unsigned)(nt * STEP_C));
+        cfg.blockDim = dim3(256);
+        cfg.dynamicSmemBytes = sizeof(c64) * (size_t)cnt;   // at most 16 KB (m <= 1024)
+        cfg.stream = s;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        LAPH_CUDA(cudaLaunchKernelEx(&cfg, lanczos_end_kernel, n, ldv, j, V, w, part, H, nrm, flag, h_vec));
         LAPH_LAUNCH_CHECK();
     }
     c64 *h_vec;
+    bool have_vec = false;   // h_vec holds the last basis vector
 };
 
 // Eigen-decomposition of the leading m x m Hermitian part of H[t] (row stride ldh) for every slice.
@@ -676,6 +754,7 @@ extern "C" int laph_eigvecs(laph_ctx *ctx, const laph_lattice *lat, const void *
         lz.h_vec = (c64 *)ws_get(ctx, "eig:x", sizeof(c64) * nt * n);
         lz.H = (c64 *)ws_get(ctx, "eig:H", sizeof(c64) * nt * (size_t)(m + 1) * (m + 1));
         lz.h = (c64 *)ws_get(ctx, "eig:h", sizeof(c64) * nt * (size_t)(m + 2));
+        lz.part = (c64 *)ws_get(ctx, "eig:hpart", sizeof(c64) * nt * STEP_C * (size_t)(m + 2));
         lz.nrm = (double *)ws_get(ctx, "eig:nrm", sizeof(double) * nt);
         lz.ca = (double *)ws_get(ctx, "eig:ca", sizeof(double) * nt);
         lz.cb = (double *)ws_get(ctx, "eig:cb", sizeof(double) * nt);
@@ -732,6 +811,7 @@ extern "C" int laph_eigvecs(laph_ctx *ctx, const laph_lattice *lat, const void *
             set_map({}, 1);
             start_vector();
             int mest = std::min(m, nv + 24);   // enough Ritz values to bound lambda_{nv+8} from above
+            lz.have_vec = false;
             for (int j = 0; j < mest; ++j) lz.step(j);
             run_jacobi(ctx, nt, mest, m + 1, lz.H, J, Yraw, Y, theta, false, s);
             LAPH_CUDA(cudaMemcpyAsync(h_theta.data(), theta, sizeof(double) * nt * mest, cudaMemcpyDeviceToHost, s));
@@ -745,6 +825,7 @@ extern "C" int laph_eigvecs(laph_ctx *ctx, const laph_lattice *lat, const void *
         // One Lanczos cycle (steps j0 .. m-1) on the current map, its Ritz vectors Vt = V Y[:, :keep]
         // and the Rayleigh quotients mu and residuals of the nv wanted ones on -Delta itself.
         auto cycle = [&](int j0) {
+            lz.have_vec = false;
             for (int j = j0; j < m; ++j) lz.step(j);
             run_jacobi(ctx, nt, m, m + 1, lz.H, J, Yraw, Y, theta, false, s);
             rotate(ctx, n, nt, m + 1, m, keep, lz.V, Y, Vt, s);
