@@ -169,27 +169,6 @@ __global__ void gemv_n_kernel(long n, int ldv, const c64 *__restrict__ V, c64 *w
     w[(long)t * n + k] -= s;
 }
 
-// nrm[t] = ||w[t]||; flag[t] = another pass needed (norm fell by more than 1/sqrt 2); accumulates h into
-// column j of H.
-__global__ void reorth_norm_kernel(long n, int ldv, const c64 *w, const c64 *h, c64 *H, int j, int cnt, double *nrm,
-                                   int *flag) {
-    __shared__ c64 sm[256];
-    int t = blockIdx.x;
-    const c64 *ww = w + (long)t * n;
-    c64 a{0, 0};
-    for (long k = threadIdx.x; k < n; k += blockDim.x) a += c64{norm2(ww[k]), 0.0};
-    c64 s = block_sum(a, sm);
-    const c64 *hh = h + (long)t * (ldv + 1);
-    c64 *Ht = H + (long)t * ldv * ldv;   // H[t][row][col], ldv x ldv
-    for (int i = threadIdx.x; i < cnt; i += blockDim.x) Ht[(long)i * ldv + j] += hh[i];
-    if (threadIdx.x == 0) {
-        double after = sqrt(s.re);
-        double before = nrm[t];
-        nrm[t] = after;
-        flag[t] = after < before * 0.7071067811865476 ? 1 : 0;
-    }
-}
-
 __global__ void norm_only_kernel(long n, const c64 *w, double *nrm) {
     __shared__ c64 sm[256];
     int t = blockIdx.x;
@@ -208,50 +187,28 @@ __device__ __forceinline__ c64 ld_l2(const c64 *p) {
     return {v.x, v.y};
 }
 
-// The end of a Lanczos step, a cluster of STEP_C blocks per slice, each with a range of the vector: the further
-// passes of the orthogonalisation for the slices whose flag asks for them (at most four), then V[j+1] = w / nrm, the
-// same into next (the operand of the next step) and H[j+1][j] = nrm.  Most steps need no further pass: as separate
-// launches the four passes, the scaling and the copy were fourteen nearly empty kernels, 40 us a step.
-// 6^3 x 8, N_v = 12, the whole call 25.3 ms (30.3); 16^3 x 32, N_v = 32: 305 ms (321).
+// The parts of a Lanczos step that touch few vectors run on a cluster of STEP_C blocks per slice, each with a range of
+// the vector, in one launch each.
 constexpr int STEP_C = 8;
-__global__ void __launch_bounds__(256) lanczos_end_kernel(long n, int ldv, int j, c64 *V, c64 *w, c64 *part, c64 *H, double *nrm,
-                                                          int *flag, c64 *next) {
-    extern __shared__ c64 esm[];   // h of this pass [j + 1]
-    __shared__ double red[8];
-    const int t = blockIdx.x / STEP_C, rank = blockIdx.x % STEP_C, cnt = j + 1;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const long per = (n + STEP_C - 1) / STEP_C, k0 = min(n, rank * per), k1 = min(n, k0 + per);
-    c64 *Vt = V + (long)t * ldv * n, *ww = w + (long)t * n, *Ht = H + (long)t * ldv * ldv;
-    c64 *pt = part + (long)t * STEP_C * (ldv + 1);   // [rank][ldv + 1], the last for the norm
-    double b = nrm[t];
-    bool again = flag[t] != 0;
-    for (int pass = 1; pass <= 4 && again; ++pass) {
-        for (int i = warp; i < cnt; i += 8) {
-            c64 a{0, 0};
-            for (long k = k0 + lane; k < k1; k += 32) a += cmul_conj(Vt[(long)i * n + k], ww[k]);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                a.re += __shfl_xor_sync(0xffffffffu, a.re, o);
-                a.im += __shfl_xor_sync(0xffffffffu, a.im, o);
-            }
-            if (lane == 0) pt[(long)rank * (ldv + 1) + i] = a;
-        }
-        cluster_barrier();
-        for (int i = threadIdx.x; i < cnt; i += 256) {
-            c64 a{0, 0};
-            for (int r = 0; r < STEP_C; ++r) a += ld_l2(pt + (long)r * (ldv + 1) + i);
-            esm[i] = a;
-            if (rank == 0) Ht[(long)i * ldv + j] += a;
-        }
-        __syncthreads();
-        double q = 0.0;
-        for (long k = k0 + threadIdx.x; k < k1; k += 256) {
-            c64 a{0, 0};
-            for (int i = 0; i < cnt; ++i) a += Vt[(long)i * n + k] * esm[i];
-            a = ww[k] - a;
-            ww[k] = a;
-            q += norm2(a);
-        }
+struct Step {
+    long n, k0, k1;
+    int ldv, rank;
+    c64 *Vt, *w, *Ht, *pt;   // this slice's; pt [STEP_C][ldv + 1], the last for the norm
+    __device__ Step(long n_, int ldv_, c64 *V, c64 *w_, c64 *H, c64 *part) : n(n_), ldv(ldv_) {
+        const int t = blockIdx.x / STEP_C;
+        rank = blockIdx.x % STEP_C;
+        const long per = (n + STEP_C - 1) / STEP_C;
+        k0 = min(n, rank * per);
+        k1 = min(n, k0 + per);
+        Vt = V + (long)t * ldv * n;
+        w = w_ + (long)t * n;
+        Ht = H + (long)t * ldv * ldv;
+        pt = part + (long)t * STEP_C * (ldv + 1);
+    }
+    // ||w|| from the threads' sums q of |w|^2
+    __device__ double norm(double q) const {
+        __shared__ double red[8];
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
         if (lane == 0) red[warp] = q;
@@ -261,19 +218,92 @@ __global__ void __launch_bounds__(256) lanczos_end_kernel(long n, int ldv, int j
             pt[(long)rank * (ldv + 1) + ldv] = c64{q, 0.0};
         }
         cluster_barrier();
-        double after = 0.0;
-        for (int r = 0; r < STEP_C; ++r) after += ld_l2(pt + (long)r * (ldv + 1) + ldv).re;
-        after = sqrt(after);
-        again = pass < 4 && after < b * 0.7071067811865476;
-        b = after;
+        double a = 0.0;
+        for (int r = 0; r < STEP_C; ++r) a += ld_l2(pt + (long)r * (ldv + 1) + ldv).re;
+        return sqrt(a);
+    }
+    // w -= sum_i V_i <V_i, w> over i0 <= i < i0 + cnt, added to column j of H; returns ||w||.  esm: cnt entries
+    __device__ double pass(int i0, int cnt, int j, c64 *esm) const {
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        // warps share a vector where there are few (then a group of `share` warps has one vector at most)
+        const int share = cnt > 4 ? 1 : cnt > 2 ? 2 : cnt > 1 ? 4 : 8;
+        for (int i = threadIdx.x; i < cnt; i += 256) esm[i] = c64{0, 0};
+        __syncthreads();
+        for (int i = warp / share; i < cnt; i += 8 / share) {
+            c64 a{0, 0};
+            for (long k = k0 + (warp % share) * 32 + lane; k < k1; k += 32 * share) a += cmul_conj(Vt[(i0 + i) * n + k], w[k]);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                a.re += __shfl_xor_sync(0xffffffffu, a.re, o);
+                a.im += __shfl_xor_sync(0xffffffffu, a.im, o);
+            }
+            if (lane == 0 && share == 1) esm[i] = a;
+            if (lane == 0 && share > 1) esm[cnt + warp] = a;
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < cnt; i += 256) {
+            c64 a = esm[i];
+            if (share > 1)
+                for (int q = 0; q < share; ++q) a += esm[cnt + i * share + q];
+            pt[(long)rank * (ldv + 1) + i] = a;
+        }
+        cluster_barrier();
+        for (int i = threadIdx.x; i < cnt; i += 256) {
+            c64 a{0, 0};
+            for (int r = 0; r < STEP_C; ++r) a += ld_l2(pt + (long)r * (ldv + 1) + i);
+            esm[i] = a;
+            if (rank == 0) Ht[(long)(i0 + i) * ldv + j] += a;
+        }
+        __syncthreads();
+        double q = 0.0;
+        for (long k = k0 + threadIdx.x; k < k1; k += 256) {
+            c64 a{0, 0};
+            for (int i = 0; i < cnt; ++i) a += Vt[(i0 + i) * n + k] * esm[i];
+            a = w[k] - a;
+            w[k] = a;
+            q += norm2(a);
+        }
+        return norm(q);
+    }
+};
+
+// The three-term recurrence: w against v_{j-1} and v_j; nrm[t] = ||w||.
+__global__ void __launch_bounds__(256) lanczos_local_kernel(long n, int ldv, int j, c64 *V, c64 *w, c64 *part, c64 *H,
+                                                            double *nrm) {
+    extern __shared__ c64 esm[];
+    const Step st(n, ldv, V, w, H, part);
+    const int i0 = max(j - 1, 0);
+    const double b = st.pass(i0, j + 1 - i0, j, esm);
+    if (st.rank == 0 && threadIdx.x == 0) nrm[blockIdx.x / STEP_C] = b;
+}
+
+// The end of a Lanczos step behind the full pass with coefficients h: h into column j of H, up to four further full
+// passes while the norm falls by more than 1/sqrt 2 in one, then V[j+1] = w / ||w||, the same into next (the operand
+// of the next step) and H[j+1][j] = ||w||.  Most steps need no further pass: as separate launches the four passes,
+// the scaling and the copy were fourteen nearly empty kernels, 40 us a step.
+// 6^3 x 8, N_v = 12, the whole call 25.3 ms (30.3); 16^3 x 32, N_v = 32: 305 ms (321); with the local pass and this norm
+// in cluster kernels too 287 ms (300), 10^3 x 12, N_v = 20: 33.9 ms (37.2).
+__global__ void __launch_bounds__(256) lanczos_end_kernel(long n, int ldv, int j, c64 *V, c64 *w, c64 *part, c64 *H,
+                                                          const c64 *h, const double *nrm, c64 *next) {
+    extern __shared__ c64 esm[];
+    const Step st(n, ldv, V, w, H, part);
+    const int t = blockIdx.x / STEP_C, cnt = j + 1;
+    if (st.rank == 0)
+        for (int i = threadIdx.x; i < cnt; i += 256) st.Ht[(long)i * ldv + j] += h[(long)t * (ldv + 1) + i];
+    double before = nrm[t], q = 0.0;
+    for (long k = st.k0 + threadIdx.x; k < st.k1; k += 256) q += norm2(st.w[k]);
+    double b = st.norm(q);
+    for (int pass = 1; pass <= 4 && b < before * 0.7071067811865476; ++pass) {
+        before = b;
+        b = st.pass(0, cnt, j, esm);
     }
     const double inv = b > 0.0 ? 1.0 / b : 0.0;
-    for (long k = k0 + threadIdx.x; k < k1; k += 256) {
-        const c64 v = inv * ww[k];
-        Vt[(long)(j + 1) * n + k] = v;
+    for (long k = st.k0 + threadIdx.x; k < st.k1; k += 256) {
+        const c64 v = inv * st.w[k];
+        st.Vt[(long)(j + 1) * n + k] = v;
         next[(long)t * n + k] = v;
     }
-    if (rank == 0 && threadIdx.x == 0 && j + 1 < ldv) Ht[(long)(j + 1) * ldv + j] = c64{b, 0.0};
+    if (st.rank == 0 && threadIdx.x == 0 && j + 1 < ldv) st.Ht[(long)(j + 1) * ldv + j] = c64{b, 0.0};
 }
 
 // V[t][j+1] = w / nrm; H[j+1][j] = nrm (when j+1 < ldv rows)
@@ -589,7 +619,6 @@ struct Lanczos {
     const c64 *U;
     c64 *V, *w, *c0, *c1, *H, *h, *part;
     double *nrm, *ca, *cb;
-    int *flag;
     int ncheb;
     ChebFix fix;
     ChebMap map;
@@ -636,22 +665,8 @@ struct Lanczos {
         prof_begin("eig_reorth", s);
         // First the three-term recurrence, against v_j and v_{j-1} alone: it takes out nearly all of w that lies
         // in the basis, so that the pass over the whole basis behind it is in most steps the only one (its norm no
-        // longer falls; the flags still call for more where it does, as behind a restart).  The passes are
+        // longer falls; where it does, as behind a restart, further passes follow).  The passes are
         // bound by the FP64 pipe and by reading V; N_v = 32 on 16^3 x 32, the whole call, 414 ms (526).
-        const int l0 = std::max(j - 1, 0), lc = cnt - l0;
-        gemv_c_kernel<<<dim3(lc, nt), 256, 0, s>>>(n, ldv, V + (long)l0 * n, w, lc, h);
-        LAPH_LAUNCH_CHECK();
-        gemv_n_kernel<<<dim3(grid_for(n, 256), nt), 256, 0, s>>>(n, ldv, V + (long)l0 * n, w, lc, h);
-        LAPH_LAUNCH_CHECK();
-        reorth_norm_kernel<<<nt, 256, 0, s>>>(n, ldv, w, h, H + (long)l0 * ldv, j, lc, nrm, flag);
-        LAPH_LAUNCH_CHECK();
-        gemv_c_kernel<<<dim3(cnt, nt), 256, 0, s>>>(n, ldv, V, w, cnt, h);
-        LAPH_LAUNCH_CHECK();
-        gemv_n_kernel<<<dim3(grid_for(n, 256), nt), 256, 0, s>>>(n, ldv, V, w, cnt, h);
-        LAPH_LAUNCH_CHECK();
-        reorth_norm_kernel<<<nt, 256, 0, s>>>(n, ldv, w, h, H, j, cnt, nrm, flag);
-        LAPH_LAUNCH_CHECK();
-        prof_end("eig_reorth", s, 0.0, 0.0);
         cudaLaunchConfig_t cfg{};
         cudaLaunchAttribute at{};
         at.id = cudaLaunchAttributeClusterDimension;
@@ -659,12 +674,20 @@ struct Lanczos {
         at.val.clusterDim.y = at.val.clusterDim.z = 1;
         cfg.gridDim = dim3((unsigned)(nt * STEP_C));
         cfg.blockDim = dim3(256);
-        cfg.dynamicSmemBytes = sizeof(c64) * (size_t)cnt;   // at most 16 KB (m <= 1024)
+        cfg.dynamicSmemBytes = sizeof(c64) * (size_t)(cnt + 8);   // at most 16.1 KB (m <= 1024)
         cfg.stream = s;
         cfg.attrs = &at;
         cfg.numAttrs = 1;
-        LAPH_CUDA(cudaLaunchKernelEx(&cfg, lanczos_end_kernel, n, ldv, j, V, w, part, H, nrm, flag, h_vec));
+        LAPH_CUDA(cudaLaunchKernelEx(&cfg, lanczos_local_kernel, n, ldv, j, V, w, part, H, nrm));
         LAPH_LAUNCH_CHECK();
+        gemv_c_kernel<<<dim3(cnt, nt), 256, 0, s>>>(n, ldv, V, w, cnt, h);
+        LAPH_LAUNCH_CHECK();
+        gemv_n_kernel<<<dim3(grid_for(n, 256), nt), 256, 0, s>>>(n, ldv, V, w, cnt, h);
+        LAPH_LAUNCH_CHECK();
+        LAPH_CUDA(cudaLaunchKernelEx(&cfg, lanczos_end_kernel, n, ldv, j, V, w, part, H, (const c64 *)h, (const double *)nrm,
+                                     h_vec));
+        LAPH_LAUNCH_CHECK();
+        prof_end("eig_reorth", s, 0.0, 0.0);
     }
     c64 *h_vec;
     bool have_vec = false;   // h_vec holds the last basis vector
@@ -682,10 +705,11 @@ static void run_jacobi(laph_ctx *ctx, int nt, int m, int ldh, const c64 *H, c64 
     const int per = (m + C - 1) / C;
     size_t shm = sizeof(double) * (512 + mm + 2 * npair) + 16 + sizeof(c64) * npair + sizeof(int) * (2 * npair + mm) + 16;
     const size_t rows = sizeof(c64) * (size_t)per * m;
-    const int in_smem = shm + rows <= 220 * 1024 ? 1 : 0;   // below the 227 KB opt-in limit per block
+    constexpr int cap = 220 * 1024;   // below the 227 KB opt-in limit per block
+    const int in_smem = shm + rows <= cap ? 1 : 0;
     if (in_smem) {
         shm += rows;
-        LAPH_CUDA(cudaFuncSetAttribute(jacobi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+        LAPH_CUDA(cudaFuncSetAttribute(jacobi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, cap));
     }
     prof_begin("eig_jacobi", s);
     cudaLaunchConfig_t cfg{};
@@ -758,7 +782,6 @@ extern "C" int laph_eigvecs(laph_ctx *ctx, const laph_lattice *lat, const void *
         lz.nrm = (double *)ws_get(ctx, "eig:nrm", sizeof(double) * nt);
         lz.ca = (double *)ws_get(ctx, "eig:ca", sizeof(double) * nt);
         lz.cb = (double *)ws_get(ctx, "eig:cb", sizeof(double) * nt);
-        lz.flag = (int *)ws_get(ctx, "eig:flag", sizeof(int) * nt);
         c64 *J = (c64 *)ws_get(ctx, "eig:J", sizeof(c64) * nt * (size_t)m * m);
         c64 *Yraw = (c64 *)ws_get(ctx, "eig:Yraw", sizeof(c64) * nt * (size_t)m * m);
         c64 *Y = (c64 *)ws_get(ctx, "eig:Y", sizeof(c64) * nt * (size_t)m * m);
@@ -798,7 +821,6 @@ extern "C" int laph_eigvecs(laph_ctx *ctx, const laph_lattice *lat, const void *
             norm_only_kernel<<<nt, 256, 0, s>>>(n, lz.w, lz.nrm);
             LAPH_LAUNCH_CHECK();
             LAPH_CUDA(cudaMemsetAsync(lz.H, 0, sizeof(c64) * nt * (size_t)(m + 1) * (m + 1), s));
-            LAPH_CUDA(cudaMemsetAsync(lz.flag, 0, sizeof(int) * nt, s));
             lanczos_next_kernel<<<dim3(grid_for(n, 256), nt), 256, 0, s>>>(n, m + 1, -1, lz.w, lz.nrm, lz.V, lz.H);
             LAPH_LAUNCH_CHECK();
         };
