@@ -6,8 +6,8 @@
 // the end): a step takes the largest exponent E of the site and its six neighbours, shifts their entries to
 // it, and does the link products (648 IMAD.WIDE a site) and the recurrence with its coefficients in
 // integers.  One thread per site: a thread per row would shift and split the 18 neighbour reals three times.
-// A step of 4^3 x 16 or 6^3 x 8 takes 6.5 us (15.1), of 10^3 x 12 7.9 (15.7), of 16^3 x 32 34 with cold caches (95); N_v = 32 on 16^3 x 32, the whole
-// call, 648 ms (859).
+// A step of 4^3 x 16 or 6^3 x 8 takes 6.5 us (15.1), of 10^3 x 12 7.9 (15.7), of 16^3 x 32 34 with cold caches
+// (95); N_v = 32 on 16^3 x 32, the whole call, 648 ms (859).
 //
 // Accuracy: entries are cut at 2^-58 of the largest in reach and sums rounded at 2^-57 of it, against
 // 2^-53 for every FP64 operation.  A site with NaN or infinities, and every site it reaches, becomes NaN.
