@@ -367,7 +367,8 @@ __global__ void __launch_bounds__(2 * BK_SITES) blocks_kernel(Geom g, const doub
                                                               double *__restrict__ clov64, double *__restrict__ cinv64,
                                                               float *__restrict__ C32wA, float *__restrict__ C32w,
                                                               int2 *__restrict__ clovfix, int2 *__restrict__ cinvfix,
-                                                              int *__restrict__ clovexp, int *__restrict__ cinvexp) {
+                                                              int *__restrict__ clovexp, int *__restrict__ cinvexp,
+                                                              int *general) {
     __shared__ double sm[BK_SITES * 73];
     __shared__ short ex[BK_SITES * 2];     // every entry of the block is below 2^ex
     __shared__ unsigned char loc[2][BK_SITES / 2];
@@ -427,6 +428,9 @@ __global__ void __launch_bounds__(2 * BK_SITES) blocks_kernel(Geom g, const doub
         uint32_t m = 0;
 #pragma unroll 4
         for (int i = 0; i < 36; ++i) m = max(m, (uint32_t)__double2hiint(o[i]) & 0x7FFFFFFFu);
+        // limbs hold neither a block with NaN or infinities (a singular block's inverse, a mass that is not finite)
+        // nor one at the lower end of the FP64 range
+        if ((m >> 20) == 0x7FF || (m != 0 && (m >> 20) < 100)) *general = 1;
         ex[is * 2 + h] = (short)max((int)(m >> 20) - 1022, -958);
     };
     if (is < ns) put();
@@ -545,10 +549,10 @@ DiracOp prepare_dirac(laph_ctx *ctx, const Geom &g, const c64 *links, double m0,
     const double cs = -0.5 * csw / xi, ct = -0.25 * csw * (1.0 + 1.0 / xi);
     if (few)
         blocks_kernel<8><<<grid_for(g.V, 8), 16, 0, s>>>(g, F, diag, cs, ct, op.clov64, op.cinv64, op.C32wA, op.C32w,
-                                                            op.clovfix, op.cinvfix, op.clovexp, op.cinvexp);
+                                                            op.clovfix, op.cinvfix, op.clovexp, op.cinvexp, flag);
     else
         blocks_kernel<32><<<grid_for(g.V, 32), 64, 0, s>>>(g, F, diag, cs, ct, op.clov64, op.cinv64, op.C32wA, op.C32w,
-                                                              op.clovfix, op.cinvfix, op.clovexp, op.cinvexp);
+                                                              op.clovfix, op.cinvfix, op.clovexp, op.cinvexp, flag);
     LAPH_LAUNCH_CHECK();
     prepare_f32_operands(ctx, op, s);
     return op;

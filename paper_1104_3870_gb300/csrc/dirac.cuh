@@ -29,7 +29,7 @@ struct DiracOp {
     int4 *Lfix = nullptr;     // [2][4][Vh][9] (re.h, re.l, im.h, im.l)
     int2 *clovfix = nullptr, *cinvfix = nullptr;   // [2][Vh][2][36]
     int *clovexp = nullptr, *cinvexp = nullptr;    // [2][Vh][2]
-    int *general = nullptr;   // [2] device flags: links not bounded by one; the operand of this hop is not finite
+    int *general = nullptr;   // [2] device flags: links or blocks that limbs do not hold; the operand of this hop is not finite
     bool weights_bounded = true;
     laph_ctx *ctx = nullptr;  // workspace of the hop's exponents
     // FP32 inner-operator operands in packed form (dslash_f32.cu)

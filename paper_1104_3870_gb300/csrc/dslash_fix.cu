@@ -12,8 +12,8 @@
 // Accuracy: an entry is cut at 2^-58 of the power of two above the largest neighbour entry and a product
 // sum rounded at 2^-57 of it, against the 2^-53 of every FP64 operation it replaces.
 //
-// Operands with NaN or infinities, links not bounded by one and hop weights >= 1 (xi <= 1/2) take the FP64
-// kernel, which is launched behind this one and returns at once otherwise.
+// Operands and clover blocks with NaN or infinities, links not bounded by one and hop weights >= 1 (xi <= 1/2)
+// take the FP64 kernel, which is launched behind this one and returns at once otherwise.
 #include "dirac.cuh"
 #include "fixed.cuh"
 
