@@ -10,7 +10,7 @@
 // a product sum keeps sum h h' and sum (h l' + l h') in 64-bit registers (three IMAD.WIDE per real
 // product; l l' is below 2^-58), and the result is rounded to 2^-56, finer than the FP64 rounding of
 // entries near 1/2 that it replaces.  Links that are not bounded this way (a row of norm above 1.001,
-// or not finite) raise a flag, and the FP64 kernel does the lattice instead.
+// or not finite) or small against the limbs' unit raise a flag, and the FP64 kernels do the lattice instead.
 //
 //   1. pack_kernel: coalesced through shared memory; L64, L32w, the limbs by site, the flag.
 //   2. field_kernel: one thread per site, plane and pair of leaves that share their outer link (five
@@ -124,14 +124,22 @@ __global__ void __launch_bounds__(256) pack_kernel(Geom g, const c64 *__restrict
         const FX a = to_fx(v.x), b = to_fx(v.y);
         fix[(long)mk * g.V + s0 + is] = make_int4(a.h, a.l, b.h, b.l);
     }
+    // Rows of norm up to one; hop weight times row or column zero or at least 2^-5: the limbs' rounding, 2^-59
+    // an entry, is then below that of an FP64 sum over it (links of size 1e-6 lost five digits).
     bool ok = true;
-    for (int e = threadIdx.x; e < 12 * ns; e += 256) {      // rows of the matrices
+    for (int e = threadIdx.x; e < 24 * ns; e += 256) {
+        const int is = e % 12, first = (e / 24) * 36 + (e % 24 < 12 ? is * 3 : (is / 3) * 9 + is % 3);
+        const int step = e % 24 < 12 ? 1 : 3;
+        const float w = (float)(is >= 9 ? hwt : hws);
         float n = 0.f;
+        uint32_t any = 0;
         for (int k = 0; k < 3; ++k) {
-            const double2 v = sm[e * 3 + k];
+            const double2 v = sm[first + k * step];
             n = fmaf((float)v.x, (float)v.x, fmaf((float)v.y, (float)v.y, n));
+            any |= ((uint32_t)__double2hiint(v.x) << 1) | (uint32_t)__double2loint(v.x) |
+                   ((uint32_t)__double2hiint(v.y) << 1) | (uint32_t)__double2loint(v.y);
         }
-        ok &= n <= 1.001f;   // false for NaN
+        ok &= (step == 3 || n <= 1.001f) && (any == 0 || w * w * n >= 0.99f / 1024);   // false for NaN
     }
     if (!ok) *flag = 1;
 }

@@ -12,7 +12,8 @@
 // Accuracy: an entry is cut at 2^-58 of the power of two above the largest neighbour entry and a product
 // sum rounded at 2^-57 of it, against the 2^-53 of every FP64 operation it replaces.
 //
-// Operands and clover blocks with NaN or infinities, links not bounded by one and hop weights >= 1 (xi <= 1/2)
+// Operands and clover blocks with NaN or infinities, links not bounded by one, links or hop weights that are
+// small against the limbs' unit (clover.cu; ordinary links up to xi = 16 are not) and hop weights >= 1 (xi <= 1/2)
 // take the FP64 kernel, which is launched behind this one and returns at once otherwise.
 #include "dirac.cuh"
 #include "fixed.cuh"
