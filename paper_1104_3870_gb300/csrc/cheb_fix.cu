@@ -46,15 +46,16 @@ __global__ void __launch_bounds__(128) cut_vec_kernel(long V3, int nvec, long to
     const long q = i / V3, x = i - q * V3;
     const double2 *f = reinterpret_cast<const double2 *>(in) + (q / nvec) * in_ts + ((q % nvec) * V3 + x) * 3;
     double2 v[3];
-    uint32_t m = 0;
+    uint32_t m = 0, low = 0;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         v[c] = __ldg(f + c);
+        low |= (uint32_t)__double2loint(v[c].x) | (uint32_t)__double2loint(v[c].y);
         m = max(m, max((uint32_t)__double2hiint(v[c].x) & 0x7FFFFFFFu, (uint32_t)__double2hiint(v[c].y) & 0x7FFFFFFFu));
     }
     const int ex = (int)(m >> 20);
     const int E = max(ex - 1022, EXP_MIN);
-    exps[i] = (short)(ex == 0x7FF ? EXP_NAN : ex == 0 ? EXP_NONE : E);
+    exps[i] = (short)(ex == 0x7FF ? EXP_NAN : (m | low) == 0 ? EXP_NONE : E);
 #pragma unroll
     for (int c = 0; c < 3; ++c) fix[(q * 3 + c) * V3 + x] = make_longlong2(cut(v[c].x, E), cut(v[c].y, E));
 }

@@ -31,16 +31,17 @@ __global__ void __launch_bounds__(256) cut_kernel(long n, int nr, const c64 *__r
     const long o = (i / nr) * 12 * nr + i % nr;
     const double2 *f = reinterpret_cast<const double2 *>(in) + o;
     double2 v[12];
-    uint32_t m = 0;
+    uint32_t m = 0, low = 0;
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
         v[k] = __ldg(f + (long)k * nr);
         m = max(m, max((uint32_t)__double2hiint(v[k].x) & 0x7FFFFFFFu, (uint32_t)__double2hiint(v[k].y) & 0x7FFFFFFFu));
+        low |= (uint32_t)__double2loint(v[k].x) | (uint32_t)__double2loint(v[k].y);
     }
     const int ex = (int)(m >> 20);
     if (ex == 0x7FF) flag[1] = 1;
     const int E = max(ex - 1022, EXP_MIN);
-    exps[i] = (short)(ex == 0 ? EXP_NONE : E);
+    exps[i] = (short)((m | low) == 0 ? EXP_NONE : E);
 #pragma unroll
     for (int k = 0; k < 12; ++k) fix[o + (long)k * nr] = make_longlong2(cut(v[k].x, E), cut(v[k].y, E));
 }

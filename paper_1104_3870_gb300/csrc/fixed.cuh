@@ -46,13 +46,16 @@ struct Acc {
 };
 
 constexpr int EXP_NONE = -2000;   // a spinor of zeros
-constexpr int EXP_MIN = -900;
+constexpr int EXP_MIN = -1021;    // every FP64 number below 2^EXP_MIN is subnormal
 
-// floor(x 2^(58 - E)), |x| < 2^E
+// x 2^(58 - E) cut towards zero, |x| < 2^E, E >= EXP_MIN
 __device__ __forceinline__ long long cut(double x, int E) {
     const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
-    const uint64_t m = fx_shr(fx_mantissa(hi, lo), 1028 + E - (int)((hi >> 20) & 0x7FFu));
-    return (long long)(m ^ (uint64_t)(int64_t)((int32_t)hi >> 31));
+    const int ex = (int)((hi >> 20) & 0x7FFu);
+    const uint32_t top = __funnelshift_l(lo, hi, 11) | (ex ? 0x80000000u : 0u);   // zeros and subnormals have no leading one
+    const uint64_t m = fx_shr((uint64_t)top << 32 | (lo << 11), 1028 + E - max(ex, 1));
+    const uint64_t s = (uint64_t)(int64_t)((int32_t)hi >> 31);
+    return (long long)((m ^ s) - s);
 }
 // t 2^-58 as limbs, |t| < 2^59, the low one in [0, 2^30)
 __device__ __forceinline__ FX limbs58(long long t) { return {(int)(t >> 30), (int)((uint32_t)t & 0x3FFFFFFFu)}; }
