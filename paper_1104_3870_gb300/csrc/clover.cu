@@ -222,7 +222,7 @@ struct Herm6 {
     c64 l[15];
 };
 
-// Gauss-Jordan inverse with partial pivoting of a packed Hermitian block (for small pivots of L D L^dag)
+// Gauss-Jordan inverse with partial pivoting of a packed Hermitian block (for blocks that are not definite)
 __device__ __noinline__ void herm6_inverse_pivoted(const double *a_in, double *out) {
     c64 a[6][6], inv[6][6];
     for (int i = 0; i < 6; ++i)
@@ -273,11 +273,14 @@ __device__ __noinline__ void herm6_inverse_pivoted(const double *a_in, double *o
         }
 }
 
-// a <- a^{-1} by L D L^dag; false where a pivot is small against the diagonal (a is then spoilt)
+// a <- a^{-1} by L D L^dag for definite blocks; false for others (a is then spoilt).  With pivots of one sign
+// no entry exceeds the largest of the diagonal and the elimination needs no pivoting; without that, a
+// diagonal of 1e-9 beside entries of 0.2 passed a bound on the pivots and cost the inverse nine digits.
 __device__ __forceinline__ bool herm6_inverse(Herm6 &a) {
     double amax = 0.0;
 #pragma unroll
     for (int i = 0; i < 6; ++i) amax = fmax(amax, fabs(a.d[i]));
+    const bool neg = a.d[0] < 0.0;
     double di[6];   // 1 / D
     bool ok = true;
 #pragma unroll
@@ -285,7 +288,7 @@ __device__ __forceinline__ bool herm6_inverse(Herm6 &a) {
         double dj = a.d[j];
 #pragma unroll
         for (int k = 0; k < j; ++k) dj = fma(-norm2(a.l[lw(j, k)]), a.d[k], dj);
-        ok &= fabs(dj) > 0.02 * amax;   // false for NaN
+        ok &= (neg ? -dj : dj) > 0.02 * amax;   // false for NaN
         a.d[j] = dj;
         di[j] = 1.0 / dj;
         c64 v[6];   // d_k conj(l_jk)
