@@ -64,7 +64,8 @@ constexpr size_t SMEM = 2 * (size_t)BUF + 1024 + 128;
 constexpr int WARPS = 20;           // 16 that cut digits and hold the sums, a warpgroup that issues the MMAs
 constexpr long long WAIT = 1LL << 31;               // about one second at the maximum SM clock
 constexpr int E_MIN = -958;                         // least exponent: subnormals stay more than 63 bits below it
-constexpr int NONFINITE = 4096;                     // exponent of a row / column with NaN or inf
+constexpr int DIRECT = 4096;      // exponent of a row / column that has to be summed in FP64: entries at an end of the range
+constexpr int NONFINITE = 8192;   // the same with NaN or inf
 
 __device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity) {
     const long long t0 = clock64();
@@ -377,8 +378,8 @@ __device__ __forceinline__ double from_fixed(long long x, long long y, int e) {
     return neg ? -v : v;
 }
 
-// Adds the K splits and hands C[z][n][c] to Op::store; a row or column with NaN or inf goes through
-// Op::direct (the plain FP64 sum, or NaN where the entry point documents that).
+// Adds the K splits and hands C[z][n][c] to Op::store; a row or column with NaN, inf or entries at an end of
+// the FP64 range goes through Op::direct (the plain FP64 sum, or NaN where the entry point documents that).
 template <class Op>
 __global__ void finish_kernel(const Op op, int ctiles, int rtiles, int splits, long tiles,
                               const longlong2 *__restrict__ part) {
@@ -390,7 +391,7 @@ __global__ void finish_kernel(const Op op, int ctiles, int rtiles, int splits, l
     const int z = (int)(tile / ((long)ctiles * rtiles)), n = rt * TN + row, col = ct * TN + c;
     if (n >= op.rows() || col >= op.cols()) return;
     const int En = op.expA(z, n), Ec = op.expB(z, col);
-    if (En >= NONFINITE || Ec >= NONFINITE) {
+    if (En >= DIRECT || Ec >= DIRECT) {
         op.store(z, n, col, op.direct(z, n, col));
         return;
     }
@@ -407,10 +408,11 @@ __global__ void finish_kernel(const Op op, int ctiles, int rtiles, int splits, l
 }
 
 // E of a row from the largest high word of its entries (sign cleared): every entry is below 2^E; 0
-// for rows of zeros, NONFINITE where an entry is not finite.
+// for rows of zeros, NONFINITE where an entry is not finite, DIRECT where the largest is below 2^E_MIN (it
+// would be cut short) or at least 2^1023 (a loader's product may overflow).
 __device__ __forceinline__ int exp_of_hi(uint32_t h) {
     const int ex = (int)(h >> 20);
-    return ex == 0x7FF ? NONFINITE : h == 0 ? 0 : max(ex - 1022, E_MIN);
+    return ex == 0x7FF ? NONFINITE : h == 0 ? 0 : ex - 1022 < E_MIN || ex == 0x7FE ? DIRECT : ex - 1022;
 }
 __device__ __forceinline__ uint32_t hi_abs(const double2 v) {
     return max((uint32_t)__double2hiint(v.x) & 0x7FFFFFFFu, (uint32_t)__double2hiint(v.y) & 0x7FFFFFFFu);

@@ -84,9 +84,15 @@ struct SinkOp {
     }
     __device__ c64 value(const Item &, const Raw &r, int j) const { return {r.v[j].x, r.v[j].y}; }
     // a non-finite input row or column gives a non-finite coefficient
-    __device__ c64 direct(int, int, int) const {
-        const double q = __longlong_as_double(0x7FF8000000000000ll);
-        return {q, q};
+    __device__ c64 direct(int t, int n, int c) const {
+        if (expA(t, n) >= xg::NONFINITE || expB(t, c) >= xg::NONFINITE) {
+            const double q = __longlong_as_double(0x7FF8000000000000ll);
+            return {q, q};
+        }
+        const c64 *a = itemA(t, n).p, *b = itemB(t, c).p;
+        c64 s{0, 0};
+        for (long k = 0; k < K; ++k) s += conj(a[k]) * b[k + 9 * (k / 3)];   // x 12 + c
+        return s;
     }
     __device__ void store(int t, int n, int c, c64 v) const { coef[(((long)(c >> 2) * nt + t) * 4 + (c & 3)) * nv + n] = v; }
 };
