@@ -1,8 +1,7 @@
 // The restart GEMM of the eigensolver, Out[t][c] = sum_{j < m} V[t][j] Y[t][j][c] for c < k, on the
 // exact-slice tensor-core GEMM (exact_gemm.cuh): rows are the entries of the vectors, K the m basis vectors.
 // Bound by the FP64 pipe in FP64 (four multiply-adds per term at two per cycle and SM); here by the start and
-// drain of short CTAs (m = 80: five sub-chunks) and the partial sums.  The slices go in passes so that those
-// stay below 512 MB.
+// drain of short CTAs (m = 80: five sub-chunks) and the partial sums.
 // 10^3 x 12, m = 56: about 70 us (1290); N_v = 32 on 16^3 x 32, the whole call, 526 ms (648).
 #include "exact_gemm.cuh"
 
@@ -79,18 +78,12 @@ __global__ void __launch_bounds__(128) strided_exp_kernel(long rows, int m, long
 void rotate_tc(laph_ctx *ctx, long n, int nt, int ldv, int m, int k, const c64 *V, const c64 *Y, c64 *out, cudaStream_t s) {
     int *EA = (int *)ws_get(ctx, "eig:expV", sizeof(int) * nt * (size_t)n);
     int *EB = (int *)ws_get(ctx, "eig:expY", sizeof(int) * nt * (size_t)k);
-    const long per_slice = ((n + xg::TN - 1) / xg::TN) * ((k + xg::TN - 1) / xg::TN) * (long)sizeof(longlong2) * 2 * xg::TN * xg::TN;
-    const int chunk = (int)std::max(1l, std::min<long>(std::min(nt, 65535), (512l << 20) / per_slice));
-    for (int t0 = 0; t0 < nt; t0 += chunk) {
-        const int c = std::min(chunk, nt - t0);
-        const c64 *v = V + (long)t0 * ldv * n, *y = Y + (long)t0 * m * m;
-        strided_exp_kernel<<<dim3(grid_for(n, 128), c), 128, 0, s>>>(n, m, n, (long)ldv * n, v, EA);
-        LAPH_LAUNCH_CHECK();
-        strided_exp_kernel<<<dim3(grid_for(k, 128), c), 128, 0, s>>>(k, m, m, (long)m * m, y, EB);
-        LAPH_LAUNCH_CHECK();
-        RotateOp op{v, y, EA, EB, n, ldv, m, k, out + (long)t0 * k * n};
-        xg::run(ctx, op, m, c, (int)n, k, s);
-    }
+    strided_exp_kernel<<<dim3(grid_for(n, 128), nt), 128, 0, s>>>(n, m, n, (long)ldv * n, V, EA);
+    LAPH_LAUNCH_CHECK();
+    strided_exp_kernel<<<dim3(grid_for(k, 128), nt), 128, 0, s>>>(k, m, m, (long)m * m, Y, EB);
+    LAPH_LAUNCH_CHECK();
+    RotateOp op{V, Y, EA, EB, n, ldv, m, k, out};
+    xg::run(ctx, op, m, nt, (int)n, k, s);
 }
 
 }  // namespace laph

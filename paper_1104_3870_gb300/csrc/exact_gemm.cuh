@@ -40,6 +40,7 @@
 // Every wait is bounded (about a second); a wait that gives up sets a host-visible flag, the CTA
 // stops issuing, waits for its issued MMAs (bounded) and frees its TMEM.
 #pragma once
+#include <algorithm>
 #include <cstdint>
 #include <type_traits>
 
@@ -134,7 +135,7 @@ __device__ __forceinline__ uint32_t digit_pair(const Fix &re, const Fix &im) {
 //   so the four lanes of a row read 64 contiguous bytes (the order of k is free as long as A and B share it)
 template <class Op>
 __global__ void __launch_bounds__(WARPS * 32, 1)
-    gemm_kernel(const Op op, int ctiles, int rtiles, int splits, int nsub, longlong2 *__restrict__ part, int *flag) {
+    gemm_kernel(const Op op, int ctiles, int rtiles, int splits, int nsub, int tile0, longlong2 *__restrict__ part, int *flag) {
     extern __shared__ unsigned char xsm[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     unsigned char *base = (unsigned char *)(((uintptr_t)xsm + 1023) & ~(uintptr_t)1023);
@@ -143,8 +144,9 @@ __global__ void __launch_bounds__(WARPS * 32, 1)
     const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(base);
     const uint32_t full0 = (uint32_t)__cvta_generic_to_shared(bars), empty0 = full0 + 16, drained = full0 + 32;
 
-    // unit: column tile fastest, then row tile, K split, batch (the CTAs of a batch share its operands in L2)
-    int u = blockIdx.x;
+    // unit: column tile fastest, then row tile, K split, batch (the CTAs of a batch share its operands in L2);
+    // a pass from tile tile0 on has one split unless it is the only one
+    int u = tile0 + blockIdx.x;
     const int ct = u % ctiles;
     u /= ctiles;
     const int rt = u % rtiles;
@@ -320,7 +322,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1)
             if (lane == 0) *(volatile int *)flag = 1;
         } else {
             // part[split][tile][column 64][real row 128]; the lane is the real row
-            const long tile = ((long)z * rtiles + rt) * ctiles + ct;
+            const long tile = ((long)z * rtiles + rt) * ctiles + ct - tile0;
             const long tiles = (long)(gridDim.x / splits);
             longlong2 *dst = part + ((split * tiles + tile) * TN + (warp >> 2) * 16) * (2 * TN) + (warp & 3) * 32 + lane;
 #pragma unroll
@@ -381,14 +383,14 @@ __device__ __forceinline__ double from_fixed(long long x, long long y, int e) {
 // Adds the K splits and hands C[z][n][c] to Op::store; a row or column with NaN, inf or entries at an end of
 // the FP64 range goes through Op::direct (the plain FP64 sum, or NaN where the entry point documents that).
 template <class Op>
-__global__ void finish_kernel(const Op op, int ctiles, int rtiles, int splits, long tiles,
+__global__ void finish_kernel(const Op op, int ctiles, int rtiles, int splits, int tile0, long tiles,
                               const longlong2 *__restrict__ part) {
     const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
     const int row = (int)(idx % TN), c = (int)((idx / TN) % TN);
-    const long tile = idx / (TN * TN);
+    const long tile = idx / (TN * TN), of = tile0 + tile;   // in the pass, of all
     if (tile >= tiles) return;
-    const int ct = (int)(tile % ctiles), rt = (int)((tile / ctiles) % rtiles);
-    const int z = (int)(tile / ((long)ctiles * rtiles)), n = rt * TN + row, col = ct * TN + c;
+    const int ct = (int)(of % ctiles), rt = (int)((of / ctiles) % rtiles);
+    const int z = (int)(of / ((long)ctiles * rtiles)), n = rt * TN + row, col = ct * TN + c;
     if (n >= op.rows() || col >= op.cols()) return;
     const int En = op.expA(z, n), Ec = op.expB(z, col);
     if (En >= DIRECT || Ec >= DIRECT) {
@@ -477,6 +479,8 @@ inline int choose_splits(long tiles, int nsub, int sms) {
 int *host_flag(laph_ctx *ctx);
 void check_host_flag(laph_ctx *ctx);
 
+constexpr long PASS = 4096;   // tiles whose partial sums are kept at a time: 512 MB
+
 template <class Op>
 void run(laph_ctx *ctx, const Op &op, long K, int nbatch, int rows, int cols, cudaStream_t s) {
     static bool attr[64] = {false};
@@ -487,14 +491,19 @@ void run(laph_ctx *ctx, const Op &op, long K, int nbatch, int rows, int cols, cu
     const int ctiles = (cols + TN - 1) / TN, rtiles = (rows + TN - 1) / TN;
     const int nsub = (int)((2 * K + KS - 1) / KS);
     const long tiles = (long)nbatch * ctiles * rtiles;
-    const int splits = choose_splits(tiles, nsub, ctx->sm_count > 0 ? ctx->sm_count : 152);
-    LAPH_REQUIRE(tiles * splits < (1L << 31), "problem too large");
-    longlong2 *part = (longlong2 *)ws_get(ctx, "xgemm:part", sizeof(longlong2) * 2 * TN * TN * (size_t)(tiles * splits));
-    gemm_kernel<Op><<<(unsigned)(tiles * splits), WARPS * 32, SMEM, s>>>(op, ctiles, rtiles, splits, nsub, part,
-                                                                       host_flag(ctx));
-    LAPH_LAUNCH_CHECK();
-    finish_kernel<Op><<<(unsigned)(tiles * (TN * TN / 256)), 256, 0, s>>>(op, ctiles, rtiles, splits, tiles, part);
-    LAPH_LAUNCH_CHECK();
+    LAPH_REQUIRE(tiles < (1L << 31), "problem too large");
+    int splits = choose_splits(tiles, nsub, ctx->sm_count > 0 ? ctx->sm_count : 152);
+    if (tiles * splits > PASS) splits = 1;   // 27 waves and more: nothing to split for
+    const size_t unit = sizeof(longlong2) * 2 * TN * TN;
+    longlong2 *part = (longlong2 *)ws_get(ctx, "xgemm:part", unit * (size_t)std::min(tiles * splits, PASS));
+    for (long t0 = 0; t0 < tiles; t0 += PASS) {
+        const long n = std::min(tiles - t0, PASS);
+        gemm_kernel<Op><<<(unsigned)(n * splits), WARPS * 32, SMEM, s>>>(op, ctiles, rtiles, splits, nsub, (int)t0, part,
+                                                                         host_flag(ctx));
+        LAPH_LAUNCH_CHECK();
+        finish_kernel<Op><<<(unsigned)(n * (TN * TN / 256)), 256, 0, s>>>(op, ctiles, rtiles, splits, (int)t0, n, part);
+        LAPH_LAUNCH_CHECK();
+    }
 }
 
 }  // namespace xg
