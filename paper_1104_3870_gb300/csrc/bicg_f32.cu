@@ -234,8 +234,10 @@ __device__ __forceinline__ void stop_rhs(const BicgScalars &sc, int k, int statu
 __global__ void __launch_bounds__(256) alpha_check_kernel(BicgScalars sc, const double *__restrict__ rr_part, int rr_count,
                                                           int nr, int first, PartSums rv, int *live) {
     __shared__ double sm[16];
-    if (*live == 0) return;
     const int r = blockIdx.x;
+    // not by *live: other blocks count it down meanwhile, and the warps of a block have to agree.  active[r] is
+    // written by this block alone, behind a barrier.
+    if (!sc.active[r]) return;
     double rr = 0.0;
     if (!first) {
         for (int i = threadIdx.x; i < rr_count; i += blockDim.x) rr += rr_part[(long)i * nr + r];
@@ -248,7 +250,7 @@ __global__ void __launch_bounds__(256) alpha_check_kernel(BicgScalars sc, const 
     }
     c64 d[1];
     if (rv.p) sum_parts<1>(rv, r, d, sm);
-    if (threadIdx.x != 0 || !sc.active[r]) return;
+    if (threadIdx.x != 0) return;
     if (!first) {
         sc.rr[r] = rr;
         const int s = sc.status[r];
