@@ -216,12 +216,22 @@ void ChebMap::set(laph_ctx *ctx, const char *name, const std::vector<double> &a,
     LAPH_CUDA(cudaMemcpyAsync(e, he.data(), sizeof(int) * nt, cudaMemcpyHostToDevice, s));
 }
 
-void ChebFix::init(laph_ctx *c, const Geom &geom, const c64 *U, cudaStream_t s) {
+void ChebFix::init(laph_ctx *c, const Geom &geom, const c64 *U, int nvec, cudaStream_t s) {
     ctx = c;
     g = geom;
     u = nullptr;
     if (g.V3 >= (1l << 30)) return;
-    int4 *w = (int4 *)ws_get(ctx, "cheb:links", sizeof(int4) * 27 * g.V);
+    // vectors of a pass: three buffers of at most 256 MB (one vector of every slice at least)
+    const size_t one = (size_t)g.V * 3 * sizeof(longlong2);
+    chunk = (int)std::max(1l, std::min<long>(nvec, (256l << 20) / (long)one));
+    longlong2 *buf = (longlong2 *)ws_spare(ctx, "cheb:f", 3 * one * chunk);
+    int4 *w = (int4 *)ws_spare(ctx, "cheb:links", sizeof(int4) * 27 * g.V);
+    if (!buf || !w) return;
+    short *exps = (short *)ws_get(ctx, "cheb:e", 3 * sizeof(short) * g.V * (size_t)chunk);
+    for (int i = 0; i < 3; ++i) {
+        f[i] = buf + (size_t)i * 3 * g.V * chunk;
+        e[i] = exps + (size_t)i * g.V * chunk;
+    }
     int *flag = (int *)ws_get(ctx, "cheb:flag", sizeof(int));
     LAPH_CUDA(cudaMemsetAsync(flag, 0, sizeof(int), s));
     links_kernel<<<grid_for(g.V, 128), 128, 0, s>>>(g.V, g.V3, U, w, flag);
@@ -234,15 +244,6 @@ void ChebFix::init(laph_ctx *c, const Geom &geom, const c64 *U, cudaStream_t s) 
 
 void ChebFix::chain(const ChebMap &m, int order, int nvec, const c64 *in, long in_ts, c64 *out, long out_ts,
                     cudaStream_t s) const {
-    // vectors of a pass: three buffers of at most 256 MB (one vector of every slice at least)
-    const long one = (long)g.nt * 3 * g.V3 * (long)sizeof(longlong2);
-    const int chunk = (int)std::max(1l, std::min<long>(nvec, (256l << 20) / one));
-    longlong2 *f[3];
-    short *e[3];
-    for (int i = 0; i < 3; ++i) {
-        f[i] = (longlong2 *)ws_get(ctx, i == 0 ? "cheb:f0" : i == 1 ? "cheb:f1" : "cheb:f2", (size_t)one * chunk);
-        e[i] = (short *)ws_get(ctx, i == 0 ? "cheb:e0" : i == 1 ? "cheb:e1" : "cheb:e2", sizeof(short) * g.V * (size_t)chunk);
-    }
     for (int v0 = 0; v0 < nvec; v0 += chunk) {
         const int nv = std::min(chunk, nvec - v0);
         const long total = (long)g.nt * nv * g.V3;

@@ -19,9 +19,13 @@ struct ChebMap {
 struct ChebFix {
     laph_ctx *ctx = nullptr;
     Geom g;
-    const int4 *u = nullptr;   // [t][k][9][V3] link limbs; null where the links are not bounded by one
-    // builds the link limbs (synchronises); they stay null for links the format does not hold
-    void init(laph_ctx *c, const Geom &geom, const c64 *U, cudaStream_t s);
+    const int4 *u = nullptr;   // [t][k][9][V3] link limbs; null where the links are not bounded by one or memory is short
+    longlong2 *f[3] = {};      // `chunk` vectors of every slice each, and their exponents
+    short *e[3] = {};
+    int chunk = 0;
+    // builds the link limbs (synchronises); they stay null for links the format does not hold.  nvec: the most
+    // vectors of a slice that a chain will get
+    void init(laph_ctx *c, const Geom &geom, const c64 *U, int nvec, cudaStream_t s);
     bool usable(const ChebMap &m) const { return u && m.ok; }
     // out = T_order(map) in for nvec vectors of every slice; vector v of slice t at base + t * tstride + v * 3 V3
     void chain(const ChebMap &m, int order, int nvec, const c64 *in, long in_ts, c64 *out, long out_ts, cudaStream_t s) const;

@@ -114,9 +114,11 @@ __global__ void __launch_bounds__(256) pack_kernel(Geom g, const c64 *__restrict
         L64[o] = c64{v.x, v.y};
         const float re = (float)v.x, im = (float)v.y;
         L32w[o] = make_float4(re, re, im, im);
-        const double w = (pm & 3) == 3 ? hwt : hws;
-        const FX a = to_fx(w * v.x), b = to_fx(w * v.y);
-        Lfix[o] = make_int4(a.h, a.l, b.h, b.l);
+        if (Lfix) {
+            const double w = (pm & 3) == 3 ? hwt : hws;
+            const FX a = to_fx(w * v.x), b = to_fx(w * v.y);
+            Lfix[o] = make_int4(a.h, a.l, b.h, b.l);
+        }
     }
     for (int e = threadIdx.x; e < 36 * ns; e += 256) {      // [mu][k][site]
         const int is = e % ns, mk = e / ns;
@@ -348,7 +350,7 @@ __device__ __forceinline__ void store_blocks(const Geom &g, const double *sm, co
                                              int *__restrict__ aexp) {
     const int nh = ns / 2;
     // limbs of a block's entries over a power of two above them
-    for (int e = threadIdx.x; e < 2 * nh * 72; e += blockDim.x) {
+    for (int e = threadIdx.x; afix && e < 2 * nh * 72; e += blockDim.x) {
         const int k = e % 72, icb = (e / 72) % nh, p = e / (72 * nh);
         const int l = loc[p][icb], E = ex[l * 2 + k / 36];
         const FX f = to_fx(scale_pow2(sm[l * 73 + k], -E));
@@ -535,13 +537,13 @@ DiracOp prepare_dirac(laph_ctx *ctx, const Geom &g, const c64 *links, double m0,
     op.cinv64 = (double *)ws_get(ctx, "dirac:cinv64", sizeof(double) * CLOV_BLOCK * 4 * g.Vh);
     op.C32w = (float *)ws_get(ctx, "dirac:C32w", sizeof(float) * 144 * 2 * g.Vh);
     op.C32wA = (float *)ws_get(ctx, "dirac:C32wA", sizeof(float) * 144 * 2 * g.Vh);
-    op.Lfix = (int4 *)ws_get(ctx, "dirac:Lfix", sizeof(int4) * 9 * 8 * g.Vh);
-    op.clovfix = (int2 *)ws_get(ctx, "dirac:clovfix", sizeof(int2) * CLOV_BLOCK * 4 * g.Vh);
-    op.cinvfix = (int2 *)ws_get(ctx, "dirac:cinvfix", sizeof(int2) * CLOV_BLOCK * 4 * g.Vh);
+    op.Lfix = (int4 *)ws_spare(ctx, "dirac:limbs", (sizeof(int4) * 9 * 8 + 2 * sizeof(int2) * CLOV_BLOCK * 4) * g.Vh);
+    op.clovfix = op.Lfix ? (int2 *)(op.Lfix + 9 * 8 * g.Vh) : nullptr;
+    op.cinvfix = op.Lfix ? op.clovfix + CLOV_BLOCK * 4 * g.Vh : nullptr;
     op.clovexp = (int *)ws_get(ctx, "dirac:clovexp", sizeof(int) * 4 * g.Vh);
     op.cinvexp = (int *)ws_get(ctx, "dirac:cinvexp", sizeof(int) * 4 * g.Vh);
     op.ctx = ctx;
-    int4 *fix = (int4 *)ws_get(ctx, "dirac:fix", sizeof(int4) * 36 * g.V);
+    int4 *fix = (int4 *)op.C32w;   // the site limbs, 576 bytes a site as C32w, which blocks_kernel writes behind their last use
     double *F = (double *)ws_get(ctx, "dirac:F", sizeof(double) * 108 * g.V);
     int *flag = (int *)ws_get(ctx, "dirac:flag", 2 * sizeof(int));
     op.general = flag;

@@ -183,6 +183,9 @@ namespace laph {
 
 // Grow-only named device buffer of the context.
 void *ws_get(laph_ctx *ctx, const std::string &name, size_t bytes);
+// The same for a buffer that only a faster path needs: null where it would take more than an eighth of the free
+// device memory, so that a call that nearly fills the device takes the path without it and is not refused.
+void *ws_spare(laph_ctx *ctx, const std::string &name, size_t bytes);
 // Pinned host scratch of at least `bytes`.
 void *pinned_get(laph_ctx *ctx, size_t bytes);
 void ctx_activate(laph_ctx *ctx);

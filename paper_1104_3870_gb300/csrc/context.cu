@@ -100,6 +100,16 @@ void *ws_get(laph_ctx *ctx, const std::string &name, size_t bytes) {
     return b.ptr;
 }
 
+void *ws_spare(laph_ctx *ctx, const std::string &name, size_t bytes) {
+    const Buf &b = ctx->ws[name];
+    if (b.bytes < bytes) {
+        size_t free_b = 0, total_b = 0;
+        LAPH_CUDA(cudaMemGetInfo(&free_b, &total_b));
+        if (bytes > (free_b + b.bytes) / 8) return nullptr;
+    }
+    return ws_get(ctx, name, bytes);
+}
+
 void *pinned_get(laph_ctx *ctx, size_t bytes) {
     if (ctx->pinned_bytes < bytes) {
         if (ctx->pinned) {

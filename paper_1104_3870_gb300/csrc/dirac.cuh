@@ -25,7 +25,7 @@ struct DiracOp {
     double *clov64 = nullptr;  // A       [2][Vh][2][36]
     double *cinv64 = nullptr;  // A^{-1}  [2][Vh][2][36]
     // fixed-point operands of the FP64 hop (dslash_fix.cu): limbs of hw_mu U, and of the clover blocks
-    // over 2^exp
+    // over 2^exp; null where device memory is short
     int4 *Lfix = nullptr;     // [2][4][Vh][9] (re.h, re.l, im.h, im.l)
     int2 *clovfix = nullptr, *cinvfix = nullptr;   // [2][Vh][2][36]
     int *clovexp = nullptr, *cinvexp = nullptr;    // [2][Vh][2]

@@ -315,8 +315,9 @@ bool hop_fix(const DiracOp &op, int p, HopMode mode, c64 *out, const c64 *in, co
              cudaStream_t s) {
     const long n = op.g.Vh * nr;
     if (!op.weights_bounded || !op.Lfix) return false;
+    longlong2 *fix = (longlong2 *)ws_spare(op.ctx, "hop:fix", sizeof(longlong2) * 12 * n);
+    if (!fix) return false;
     short *exps = (short *)ws_get(op.ctx, "hop:exps", sizeof(short) * n);
-    longlong2 *fix = (longlong2 *)ws_get(op.ctx, "hop:fix", sizeof(longlong2) * 12 * n);
     LAPH_CUDA(cudaMemsetAsync(op.general + 1, 0, sizeof(int), s));
     cut_kernel<<<grid_for(n, 256), 256, 0, s>>>(n, nr, in, fix, exps, op.general);
     LAPH_LAUNCH_CHECK();

@@ -791,7 +791,9 @@ extern "C" int laph_eigvecs(laph_ctx *ctx, const laph_lattice *lat, const void *
         double *mu = (double *)ws_get(ctx, "eig:mu", sizeof(double) * nt * nv);
         double *res = (double *)ws_get(ctx, "eig:res", sizeof(double) * nt * nv);
         std::vector<double> ha(nt), hb(nt);
-        lz.fix.init(ctx, g, U, s);
+        int keep = std::min(m - 12, std::max(nv, nv + (m - nv) / 2));
+        keep = std::max(keep, nv);
+        lz.fix.init(ctx, g, U, keep, s);
         ChebMap unit;   // -Delta itself
         unit.set(ctx, "cheb:unit", std::vector<double>(nt, 1.0), std::vector<double>(nt, 0.0), s);
         auto set_map = [&](const std::vector<double> &lamC, int order) {
@@ -841,8 +843,6 @@ extern "C" int laph_eigvecs(laph_ctx *ctx, const laph_lattice *lat, const void *
             int idx = std::min(nv + 8, mest - 1);
             for (int t = 0; t < nt; ++t) lamC[t] = std::min(-h_theta[(size_t)t * mest + idx], 0.8 * lamL);
         }
-        int keep = std::min(m - 12, std::max(nv, nv + (m - nv) / 2));
-        keep = std::max(keep, nv);
         std::vector<double> h_res((size_t)nt * nv), h_mu((size_t)nt * nv);
         // One Lanczos cycle (steps j0 .. m-1) on the current map, its Ritz vectors Vt = V Y[:, :keep]
         // and the Rayleigh quotients mu and residuals of the nv wanted ones on -Delta itself.

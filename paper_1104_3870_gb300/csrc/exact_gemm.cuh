@@ -479,7 +479,8 @@ inline int choose_splits(long tiles, int nsub, int sms) {
 int *host_flag(laph_ctx *ctx);
 void check_host_flag(laph_ctx *ctx);
 
-constexpr long PASS = 4096;   // tiles whose partial sums are kept at a time: 512 MB
+// Tiles whose partial sums are kept at a time: 512 MB, 27 waves of CTAs; down to 32 MB where device memory is short
+constexpr long PASS = 4096, PASS_MIN = 256;
 
 template <class Op>
 void run(laph_ctx *ctx, const Op &op, long K, int nbatch, int rows, int cols, cudaStream_t s) {
@@ -493,11 +494,14 @@ void run(laph_ctx *ctx, const Op &op, long K, int nbatch, int rows, int cols, cu
     const long tiles = (long)nbatch * ctiles * rtiles;
     LAPH_REQUIRE(tiles < (1L << 31), "problem too large");
     int splits = choose_splits(tiles, nsub, ctx->sm_count > 0 ? ctx->sm_count : 152);
-    if (tiles * splits > PASS) splits = 1;   // 27 waves and more: nothing to split for
     const size_t unit = sizeof(longlong2) * 2 * TN * TN;
-    longlong2 *part = (longlong2 *)ws_get(ctx, "xgemm:part", unit * (size_t)std::min(tiles * splits, PASS));
-    for (long t0 = 0; t0 < tiles; t0 += PASS) {
-        const long n = std::min(tiles - t0, PASS);
+    long pass = std::min(tiles * splits, PASS);
+    longlong2 *part = nullptr;
+    while (pass > PASS_MIN && !(part = (longlong2 *)ws_spare(ctx, "xgemm:part", unit * (size_t)pass))) pass = std::max(pass / 2, PASS_MIN);
+    if (!part) part = (longlong2 *)ws_get(ctx, "xgemm:part", unit * (size_t)pass);
+    if (pass < tiles * splits) splits = 1;
+    for (long t0 = 0; t0 < tiles; t0 += pass) {
+        const long n = std::min(tiles - t0, pass);
         gemm_kernel<Op><<<(unsigned)(n * splits), WARPS * 32, SMEM, s>>>(op, ctiles, rtiles, splits, nsub, (int)t0, part,
                                                                          host_flag(ctx));
         LAPH_LAUNCH_CHECK();
