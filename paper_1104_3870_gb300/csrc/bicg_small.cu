@@ -7,9 +7,9 @@
 // four partial sums are exchanged by shuffles, and lane mu forms the three components of spin mu.  A
 // lane keeps its components of x, r, p, v, s and t in registers; only the operand of the next hop leaves
 // it, through the shared memory of its CTA, which the cluster reads, between cluster barriers (six an
-// iteration).  Inner products are
-// compensated FP32 sums (two floats, 48 bits), over lanes, warps and CTAs in a fixed order, so every
-// CTA of a cluster takes the same decision.
+// iteration).  Inner products are FP32 products in two-float sums (48 bits), over lanes, warps and CTAs in
+// a fixed order, so every CTA of a cluster takes the same decision; their error is the rounding of the
+// products, 2^-24 as in the streamed solver.
 //
 // The recurrences are those of solver.cu with the coded shadow vector of blas.cuh, with two changes
 // that save a barrier: <rhat, r> of the new residual is <rhat, s> - omega <rhat, t>, and <r, r> is summed

@@ -9,8 +9,8 @@
 // A step of 4^3 x 16 or 6^3 x 8 takes 6.5 us (15.1), of 10^3 x 12 7.9 (15.7), of 16^3 x 32 34 with cold caches
 // (95); N_v = 32 on 16^3 x 32, the whole call, 648 ms (859).
 //
-// Accuracy: entries are cut at 2^-58 of the largest in reach and sums rounded at 2^-57 of it, against
-// 2^-53 for every FP64 operation.  A site with NaN or infinities, and every site it reaches, becomes NaN.
+// Accuracy: entries are cut at 2^-58 of the largest in reach and sums rounded at 2^-57 of it, with the products of
+// low limbs left out (rms 2^-57.3 a sum), against 2^-53 for every FP64 operation.  A site with NaN or infinities, and every site it reaches, becomes NaN.
 #include <cmath>
 
 #include "cheb_fix.cuh"

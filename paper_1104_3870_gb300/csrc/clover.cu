@@ -8,7 +8,7 @@
 // point on the integer pipe (64 multiply-adds per cycle and SM): a real is two limbs,
 //   x = h 2^-28 + l 2^-58,  |l| <= 2^29,
 // a product sum keeps sum h h' and sum (h l' + l h') in 64-bit registers (three IMAD.WIDE per real
-// product; l l' is below 2^-58), and the result is rounded to 2^-56, finer than the FP64 rounding of
+// product; l l', below 2^-58, is left out), and the result is rounded to 2^-56, finer than the FP64 rounding of
 // entries near 1/2 that it replaces.  Links that are not bounded this way (a row of norm above 1.001,
 // or not finite) or small against the limbs' unit raise a flag, and the FP64 kernels do the lattice instead.
 //

@@ -203,8 +203,9 @@ __global__ void __launch_bounds__(256) hop_kernel(DiracOp op, int p, cpx<T> *__r
 // Algorithmic traffic of one hop launch over the Vh output sites of a parity:
 // each neighbour spinor is read once per launch (24 reals), the output written
 // once (24 reals), the xpay/residual operands read once (24 reals each); the 8
-// links touching a site are read once per launch (12 reals compressed for FP32,
-// 18 for FP64) and the clover block once (72 reals).
+// links touching a site are read once per launch (18 reals for FP64; for FP32 the 12
+// that an SU(3) matrix needs, although the FP32 kernels read 3x3 links with every real
+// stored twice) and the clover block once (72 reals).
 double hop_bytes(const DiracOp &op, HopMode mode, int nr, size_t real_bytes) {
     double spin = 24.0 * real_bytes;
     double per_rhs = 2.0 * spin + (mode == HOP_CLOVINV ? 0.0 : spin) + (mode == HOP_RESID || mode == HOP_APPLY ? spin : 0.0);

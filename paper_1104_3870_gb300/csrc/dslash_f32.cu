@@ -641,14 +641,14 @@ void hop_f32(const DiracOp &op, int p, HopMode mode, c32 *out, const c32 *in, co
                 : hop3_modes<2, 1>(op, p, mode, hws, hwt, o, i, zz, nr, s, live);
     } else {
         if (mode == HOP_APPLY)
-        hop2_kernel<HOP_APPLY><<<grid, block, 0, s>>>(op.nbr, op.L32w, op.C32wA, op.g.Vh, p, hws, hwt, (float2 *)out,
-                                                      (const float2 *)in, (const float2 *)z, nr, live);
-    else if (mode == HOP_CLOVINV)
-        hop2_kernel<HOP_CLOVINV><<<grid, block, 0, s>>>(op.nbr, op.L32w, op.C32w, op.g.Vh, p, hws, hwt, (float2 *)out,
-                                                        (const float2 *)in, (const float2 *)z, nr, live);
-    else
-        hop2_kernel<HOP_CLOVINV_XPAY><<<grid, block, 0, s>>>(op.nbr, op.L32w, op.C32w, op.g.Vh, p, hws, hwt,
-                                                             (float2 *)out, (const float2 *)in, (const float2 *)z, nr, live);
+            hop2_kernel<HOP_APPLY><<<grid, block, 0, s>>>(op.nbr, op.L32w, op.C32wA, op.g.Vh, p, hws, hwt, (float2 *)out,
+                                                          (const float2 *)in, (const float2 *)z, nr, live);
+        else if (mode == HOP_CLOVINV)
+            hop2_kernel<HOP_CLOVINV><<<grid, block, 0, s>>>(op.nbr, op.L32w, op.C32w, op.g.Vh, p, hws, hwt, (float2 *)out,
+                                                            (const float2 *)in, (const float2 *)z, nr, live);
+        else
+            hop2_kernel<HOP_CLOVINV_XPAY><<<grid, block, 0, s>>>(op.nbr, op.L32w, op.C32w, op.g.Vh, p, hws, hwt,
+                                                                 (float2 *)out, (const float2 *)in, (const float2 *)z, nr, live);
         LAPH_LAUNCH_CHECK();
     }
     prof_end("dslash_fp32", s, hop_bytes(op, mode, nr, sizeof(float)), hop_flops(op, nr));

@@ -15,7 +15,8 @@
 // wanted N_v are checked explicitly on -Delta itself.
 //
 // All slices advance together (the slice is the batch index); every array has
-// a leading slice dimension.  FP64 throughout.
+// a leading slice dimension.  FP64 but for the Chebyshev chain (two-limb fixed point, cheb_fix.cu) and the
+// basis rotations (exact slices on the tensor cores, eig_rotate_tc.cu).
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -281,8 +282,8 @@ __global__ void __launch_bounds__(256) lanczos_local_kernel(long n, int ldv, int
 // passes while the norm falls by more than 1/sqrt 2 in one, then V[j+1] = w / ||w||, the same into next (the operand
 // of the next step) and H[j+1][j] = ||w||.  Most steps need no further pass: as separate launches the four passes,
 // the scaling and the copy were fourteen nearly empty kernels, 40 us a step.
-// 6^3 x 8, N_v = 12, the whole call 25.3 ms (30.3); 16^3 x 32, N_v = 32: 305 ms (321); with the local pass and this norm
-// in cluster kernels too 287 ms (300), 10^3 x 12, N_v = 20: 33.9 ms (37.2).
+// 6^3 x 8, N_v = 12, the whole call 25.3 ms (30.3); 16^3 x 32, N_v = 32: 16 ms less; with the local pass and this norm
+// in cluster kernels too another 13 ms less (286 to 297 ms in all, by box), 10^3 x 12, N_v = 20: 33.9 ms (37.2).
 __global__ void __launch_bounds__(256) lanczos_end_kernel(long n, int ldv, int j, c64 *V, c64 *w, c64 *part, c64 *H,
                                                           const c64 *h, const double *nrm, c64 *next) {
     extern __shared__ c64 esm[];
@@ -306,22 +307,13 @@ __global__ void __launch_bounds__(256) lanczos_end_kernel(long n, int ldv, int j
     if (st.rank == 0 && threadIdx.x == 0 && j + 1 < ldv) st.Ht[(long)(j + 1) * ldv + j] = c64{b, 0.0};
 }
 
-// V[t][j+1] = w / nrm; H[j+1][j] = nrm (when j+1 < ldv rows)
-__global__ void lanczos_next_kernel(long n, int ldv, int j, const c64 *w, const double *nrm, c64 *V, c64 *H) {
+// V[t][0] = w / nrm
+__global__ void lanczos_start_kernel(long n, int ldv, const c64 *w, const double *nrm, c64 *V) {
     int t = blockIdx.y;
     long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
     double b = nrm[t];
     double inv = b > 0.0 ? 1.0 / b : 0.0;
-    if (k < n) V[((long)t * ldv + j + 1) * n + k] = inv * w[(long)t * n + k];
-    if (k == 0 && j >= 0 && j + 1 < ldv) H[(long)t * ldv * ldv + (long)(j + 1) * ldv + j] = c64{b, 0.0};
-}
-
-__global__ void scale_kernel(long n, c64 *v, const double *nrm) {
-    int t = blockIdx.y;
-    long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    double b = nrm[t];
-    v[(long)t * n + k] = (b > 0.0 ? 1.0 / b : 0.0) * v[(long)t * n + k];
+    if (k < n) V[(long)t * ldv * n + k] = inv * w[(long)t * n + k];
 }
 
 // ------------------------------------------------------------------ batched complex Jacobi
@@ -823,7 +815,7 @@ extern "C" int laph_eigvecs(laph_ctx *ctx, const laph_lattice *lat, const void *
             norm_only_kernel<<<nt, 256, 0, s>>>(n, lz.w, lz.nrm);
             LAPH_LAUNCH_CHECK();
             LAPH_CUDA(cudaMemsetAsync(lz.H, 0, sizeof(c64) * nt * (size_t)(m + 1) * (m + 1), s));
-            lanczos_next_kernel<<<dim3(grid_for(n, 256), nt), 256, 0, s>>>(n, m + 1, -1, lz.w, lz.nrm, lz.V, lz.H);
+            lanczos_start_kernel<<<dim3(grid_for(n, 256), nt), 256, 0, s>>>(n, m + 1, lz.w, lz.nrm, lz.V);
             LAPH_LAUNCH_CHECK();
         };
         std::vector<double> h_theta((size_t)nt * m);

@@ -15,7 +15,8 @@
 // cores' FP32 accumulation is exact.  The eight diagonals D = 2..9 (36 digit pairs) are read from
 // TMEM every 512 real k and added as integers into one 96-bit sum per output (units of 2^-61), which
 // stays exact too; splitting K over CTAs adds such sums, so a result does not depend on the split.  What is lost: the rounding of the entries
-// (2^-56 of the largest entry of the row or column) and the pairs j + l >= 10 (seven products of
+// (2^-56 of the largest entry of the row or column, so an entry below an eighth of that keeps fewer than 53
+// bits, and a result is accurate to the rows' largest entries, not to its own size) and the pairs j + l >= 10 (seven products of
 // at most 2^-56 each at D = 10).  With x of typical size 1/20 of the row's largest entry that is
 // below the rounding of an FP64 sum.
 //

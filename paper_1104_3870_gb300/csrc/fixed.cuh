@@ -1,7 +1,8 @@
 // Two-limb fixed-point arithmetic on the integer pipe, for FP64-accurate products of bounded numbers on
 // a GPU with two FP64 multiply-adds per cycle and SM.  A real is x = h 2^-28 + l 2^-58 with |l| <= 2^29;
 // a product sum keeps sum h h' and sum (h l' + l h') in 64-bit registers (three IMAD.WIDE per real
-// product; l l' is below 2^-58).
+// product).  l l' is left out: below 2^-58 for two such limbs, below 2^-57 where one comes from limbs58 (a low
+// limb in [0, 2^30)), with an rms of 2^-57.3 for the six of a row times a vector.
 #pragma once
 #include "common.cuh"
 

@@ -28,12 +28,6 @@ inline Mat4 mat_dag(const Mat4 &a) {
         for (int j = 0; j < 4; ++j) r.m[i][j] = conj(a.m[j][i]);
     return r;
 }
-inline Mat4 mat_scale(double s, const Mat4 &a) {
-    Mat4 r;
-    for (int i = 0; i < 4; ++i)
-        for (int j = 0; j < 4; ++j) r.m[i][j] = s * a.m[i][j];
-    return r;
-}
 // chiral basis: gamma_mu = [[0, G], [G^dag, 0]], G_k = -i sigma_k, G_4 = 1
 inline Mat4 gamma_mat(int mu) {
     const c64 O{0, 0}, P{1, 0}, M1{-1, 0}, I{0, 1}, Mi{0, -1};
