@@ -71,19 +71,22 @@ std::vector<uint8_t> dilution_masks(const laph_dilution &d, int nt, int nv, cons
 // out[b][site][alpha][c] = (gamma_4 y)_alpha,  y_alpha = sum_n V(t,n,x,c) [P^(b) rho](t,alpha,n).
 // gamma_4 swaps the upper and lower spin pairs (chiral basis).
 //
-// Bound by the store of the result.  A block writes SRC_SITES sites of one slice and projector: zeros in
+// Bound by the store of the result.  A block writes `sites` sites of one slice and projector: zeros in
 // contiguous 16-byte stores where the time projector leaves the slice out (15 of 16 slices of (TI16, .)),
-// else through shared memory, from where they leave contiguously too.  (One thread per site and colour,
-// storing four 16-byte pieces 48 bytes apart, reached 73 % of the copy bandwidth: half sectors.)
-// 24^3 x 128, N_v = 64, 32 sources: 1.94 ms, 93 % of the copy bandwidth (2.48 ms).
-constexpr int SRC_SITES = 512, SRC_TILE = 64, SRC_THREADS = 192;
-__global__ void __launch_bounds__(SRC_THREADS) sources_kernel(long V3, int nt, int nv, int chunks, const c64 *__restrict__ evecs,
+// else tile by tile through shared memory, from where they leave contiguously too.  (One thread per site and
+// colour, storing four 16-byte pieces 48 bytes apart, reached 73 % of the copy bandwidth: half sectors.)  The
+// vectors that the projector holds are listed once, so that a thread has eight of their entries in flight.
+// 24^3 x 128, N_v = 64, 32 sources: 1.87 ms, 97 % of the copy bandwidth (1.92 ms without the list, 2.48 ms with one
+// thread per site and colour); 12^3 x 16, 32 of 64 vectors in each of 16 sources: 185 us (338 and 201).
+constexpr int SRC_SITES = 512, SRC_TILE = 64, SRC_THREADS = 192, SRC_LIST = 192;
+__global__ void __launch_bounds__(SRC_THREADS) sources_kernel(long V3, int nt, int nv, int chunks, int sites,
+                                                              const c64 *__restrict__ evecs,
                                                               const uint8_t *__restrict__ codes,
                                                               const uint8_t *__restrict__ mask, c64 *__restrict__ out) {
     const unsigned u = blockIdx.x / (unsigned)chunks, b = u / (unsigned)nt;   // (projector, slice)
     const int t = (int)(u - b * nt);
-    const long x0 = (long)(blockIdx.x - u * chunks) * SRC_SITES;
-    const int ns = (int)min((long)SRC_SITES, V3 - x0);
+    const long x0 = (long)(blockIdx.x - u * chunks) * sites;
+    const int ns = (int)min((long)sites, V3 - x0);
     const uint8_t *m = mask + (long)b * (nt + 4 + nv);
     double2 *o = reinterpret_cast<double2 *>(out) + ((long)u * V3 + x0) * 12;
     if (!m[t]) {
@@ -92,31 +95,78 @@ __global__ void __launch_bounds__(SRC_THREADS) sources_kernel(long V3, int nt, i
         return;
     }
     __shared__ double2 sm[SRC_TILE * 12];
-    const int is = threadIdx.x / 3, c = threadIdx.x % 3;
+    __shared__ unsigned list[SRC_LIST];   // the projector's n among SRC_LIST, ascending: n << 8 | four 2-bit codes
+    __shared__ int held[SRC_THREADS / 32];
+    const int is = threadIdx.x / 3, c = threadIdx.x % 3, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool on[4] = {m[nt] != 0, m[nt + 1] != 0, m[nt + 2] != 0, m[nt + 3] != 0};
+    auto build = [&](int n0) {
+        const int n = n0 + (int)threadIdx.x;
+        const bool in = n < nv && m[nt + 4 + n];
+        unsigned w = (unsigned)n << 8;
+        if (n < nv)
+            for (int a = 0; a < 4; ++a) w |= (unsigned)codes[(t * 4 + a) * nv + n] << (2 * a);
+        const unsigned who = __ballot_sync(0xffffffffu, in);
+        if (lane == 0) held[warp] = __popc(who);
+        __syncthreads();
+        int first = 0, cnt = 0;
+        for (int q = 0; q < SRC_THREADS / 32; ++q) {
+            if (q < warp) first += held[q];
+            cnt += held[q];
+        }
+        if (in) list[first + __popc(who & ((1u << lane) - 1))] = w;
+        __syncthreads();
+        return cnt;
+    };
+    int cnt = build(0);
     for (int s0 = 0; s0 < ns; s0 += SRC_TILE) {
         const int tile = min(SRC_TILE, ns - s0);
         c64 y[4] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
-        if (is < tile) {
+        for (int n0 = 0; n0 < nv; n0 += SRC_LIST) {
+            if (nv > SRC_LIST && n0 + s0 > 0) {   // more vectors than a list holds
+                __syncthreads();
+                cnt = build(n0);
+            }
+            if (is >= tile) continue;
             const c64 *v = evecs + ((long)t * nv * V3 + x0 + s0 + is) * 3 + c;
-            for (int n = 0; n < nv; ++n) {
-                if (!m[nt + 4 + n]) continue;
-                const c64 vn = v[(long)n * V3 * 3];
+            for (int i0 = 0; i0 < cnt; i0 += 8) {
+                c64 vn[8];
 #pragma unroll
-                for (int a = 0; a < 4; ++a) {
-                    if (!on[a]) continue;
-                    const int code = codes[(t * 4 + a) * nv + n];
-                    // i^code * vn
-                    y[a] += code == 0 ? vn : code == 1 ? times_i(vn) : code == 2 ? -vn : -times_i(vn);
+                for (int i = 0; i < 8; ++i)
+                    if (i0 + i < cnt) vn[i] = v[(long)(list[i0 + i] >> 8) * V3 * 3];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    if (i0 + i >= cnt) break;
+                    const unsigned w = list[i0 + i];
+#pragma unroll
+                    for (int a = 0; a < 4; ++a) {
+                        if (!on[a]) continue;
+                        const unsigned code = (w >> (2 * a)) & 3u;
+                        // i^code * vn
+                        y[a] += code == 0 ? vn[i] : code == 1 ? times_i(vn[i]) : code == 2 ? -vn[i] : -times_i(vn[i]);
+                    }
                 }
             }
+        }
+        if (is < tile)
 #pragma unroll
             for (int a = 0; a < 4; ++a) sm[is * 12 + a * 3 + c] = make_double2(y[(a + 2) & 3].re, y[(a + 2) & 3].im);
-        }
         __syncthreads();
         for (int e = threadIdx.x; e < tile * 12; e += SRC_THREADS) o[s0 * 12 + e] = sm[e];
         __syncthreads();
     }
+}
+
+// Sites of a block: 512 where that leaves every SM sixteen blocks with work, else down to one tile, since
+// the tiles of a block follow one another (10^3 x 48, two sources: 39 us a call, 60 in blocks of 512 sites).
+static int sources_sites(const laph_ctx *ctx, const Geom &g, const std::vector<uint8_t> &m, int nv, int nb) {
+    long active = 0;   // (projector, slice) pairs that are not zero
+    for (int b = 0; b < nb; ++b) {
+        const uint8_t *q = m.data() + (size_t)b * (g.nt + 4 + nv);
+        active += std::count(q, q + g.nt, (uint8_t)1);
+    }
+    int sites = SRC_SITES;
+    while (sites > SRC_TILE && active * ((g.V3 + sites - 1) / sites) < 16l * (ctx->sm_count > 0 ? ctx->sm_count : 152)) sites /= 2;
+    return sites;
 }
 
 }  // namespace laph
@@ -152,12 +202,13 @@ extern "C" int laph_make_sources(laph_ctx *ctx, const laph_lattice *lat, const v
         size_t obytes = sizeof(c64) * 12 * g.V * (size_t)nb;
         StagedOut o = stage_out(ctx, rhs, obytes, "sources");
         if (nb) {
-            const int chunks = (int)((g.V3 + SRC_SITES - 1) / SRC_SITES);
+            const int sites = sources_sites(ctx, g, m, nv, nb);
+            const int chunks = (int)((g.V3 + sites - 1) / sites);
             const int per = (int)std::max(1l, std::min<long>(nb, (1l << 30) / ((long)chunks * g.nt)));   // projectors a launch
             for (int b = 0; b < nb; b += per) {
                 const int n = std::min(per, nb - b);
                 sources_kernel<<<(unsigned)((long)chunks * g.nt * n), SRC_THREADS, 0, s>>>(
-                    g.V3, g.nt, nv, chunks, ev, codes, dm + (size_t)b * (g.nt + 4 + nv), (c64 *)o.dev + (size_t)b * g.V * 12);
+                    g.V3, g.nt, nv, chunks, sites, ev, codes, dm + (size_t)b * (g.nt + 4 + nv), (c64 *)o.dev + (size_t)b * g.V * 12);
                 LAPH_LAUNCH_CHECK();
             }
         }
