@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(256) lanczos_local_kernel(long n, int ldv, int
 // of the next step) and H[j+1][j] = ||w||.  Most steps need no further pass: as separate launches the four passes,
 // the scaling and the copy were fourteen nearly empty kernels, 40 us a step.
 // 6^3 x 8, N_v = 12, the whole call 25.3 ms (30.3); 16^3 x 32, N_v = 32: 16 ms less; with the local pass and this norm
-// in cluster kernels too another 13 ms less (286 to 297 ms in all, by box), 10^3 x 12, N_v = 20: 33.9 ms (37.2).
+// in cluster kernels too another 13 ms less (286 to 297 ms in all, from GPU to GPU), 10^3 x 12, N_v = 20: 33.9 ms (37.2).
 __global__ void __launch_bounds__(256) lanczos_end_kernel(long n, int ldv, int j, c64 *V, c64 *w, c64 *part, c64 *H,
                                                           const c64 *h, const double *nrm, c64 *next) {
     extern __shared__ c64 esm[];
